@@ -379,10 +379,8 @@ __global__ void __launch_bounds__(W * 32, 2) k_band2d(const BandParams<T> p) {
           const T lL = from_left(lo_c), lR = from_right(lo_c);
 #pragma unroll
           for (int c = 0; c < NC; ++c) {
-            mx[c] = maxv(maxv(maxv(hi_c[c], hi_m[c]), maxv(hi_p[c], left_of(hi_c, c, hL))),
-                         right_of(hi_c, c, hR));
-            mn[c] = minv(minv(minv(lo_c[c], lo_m[c]), minv(lo_p[c], left_of(lo_c, c, lL))),
-                         right_of(lo_c, c, lR));
+            mx[c] = max3(max3(hi_c[c], hi_m[c], hi_p[c]), left_of(hi_c, c, hL), right_of(hi_c, c, hR));
+            mn[c] = min3(min3(lo_c[c], lo_m[c], lo_p[c]), left_of(lo_c, c, lL), right_of(lo_c, c, lR));
           }
           tape_row(5, b, mx);
           tape_row(6, b, mn);
@@ -407,9 +405,10 @@ __global__ void __launch_bounds__(W * 32, 2) k_band2d(const BandParams<T> p) {
           const T ou = ((Fp0 - nFp0) - (Fm0 - pFm0)) + ((Fp1 - nFp1) - (Fm1 - pFm1));
           const T Gi = NUG ? g_b[c] : T(1);
           const T q = q_c[c];
-          // min(1, x / |s|) is 1 for s = 0 (x/0 is inf or NaN, and min ignores NaN)
-          bun[c] = min1(fdiv(Gi * posp(mx[c] - q), absv(in)));
-          bdn[c] = min1(fdiv(Gi * posp(q - mn[c]), absv(ou)));
+          // mx - q and q - mn are never negative (q is one of the candidates); min(1, x / |s|)
+          // is 1 for s = 0 (x/0 is inf or NaN, and min ignores NaN)
+          bun[c] = min1(fdiv(Gi * (mx[c] - q), absv(in)));
+          bdn[c] = min1(fdiv(Gi * (q - mn[c]), absv(ou)));
         }
         sts(mid_row(s_bu, b), bun);
         sts(mid_row(s_bd, b), bdn);

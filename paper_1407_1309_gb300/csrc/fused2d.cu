@@ -298,10 +298,8 @@ __device__ __forceinline__ void march_tile(const F2Params<T>& p, const int strip
         T nbu[NC], nbd[NC], tmx[NC], tmn[NC];
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
-          const T mx = maxv(maxv(maxv(hi[1][c], hi[0][c]), maxv(hi[2][c], left_of(hi[1], c, hL))),
-                            right_of(hi[1], c, hR));
-          const T mn = minv(minv(minv(lo[1][c], lo[0][c]), minv(lo[2][c], left_of(lo[1], c, lL))),
-                            right_of(lo[1], c, lR));
+          const T mx = max3(max3(hi[1][c], hi[0][c], hi[2][c]), left_of(hi[1], c, hL), right_of(hi[1], c, hR));
+          const T mn = min3(min3(lo[1][c], lo[0][c], lo[2][c]), left_of(lo[1], c, lL), right_of(lo[1], c, lR));
           const T Fm0 = u0[0][c], Fp0 = u0[1][c];
           const T Fp1 = u1[1][c], Fm1 = left_of(u1[1], c, u1L);
           // [x]- = x - [x]+ and [x]+ = x - [x]- hold exactly in floating point, so the
@@ -311,9 +309,10 @@ __device__ __forceinline__ void march_tile(const F2Params<T>& p, const int strip
           const T ou = ((Fp0 - nFp0) - (Fm0 - pFm0)) + ((Fp1 - nFp1) - (Fm1 - pFm1));
           const T Gi = NUG ? gg[1][c] : T(1);
           const T q = p1[2][c];
-          // min(1, x / |s|) is 1 for s = 0 (x/0 is inf or NaN, and min ignores NaN)
-          nbu[c] = min1(fdiv(Gi * posp(mx - q), absv(in)));
-          nbd[c] = min1(fdiv(Gi * posp(q - mn), absv(ou)));
+          // mx - q and q - mn are never negative (q is one of the candidates); min(1, x / |s|)
+          // is 1 for s = 0 (x/0 is inf or NaN, and min ignores NaN)
+          nbu[c] = min1(fdiv(Gi * (mx - q), absv(in)));
+          nbd[c] = min1(fdiv(Gi * (q - mn), absv(ou)));
           tmx[c] = mx;
           tmn[c] = mn;
         }

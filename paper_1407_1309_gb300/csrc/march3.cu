@@ -112,11 +112,10 @@ __device__ __forceinline__ void put(float* dst, const float (&v)[NC]) {
   else *reinterpret_cast<float2*>(dst) = make_float2(v[0], v[1]);
 }
 
-__device__ __forceinline__ float frac1(float n, float d) { return divisible(d) ? __fdividef(n, d) : 0.0f; }
+__device__ __forceinline__ float frac1(float n, float d) { return divisible(d) ? fdiv(n, d) : 0.0f; }
 // n1/d and n2/d with one guard and one approximate reciprocal (0 when d == 0)
 __device__ __forceinline__ void frac2v(float n1, float n2, float d, float& r1, float& r2) {
-  float r;
-  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(d));
+  const float r = rcp(d);
   r1 = divisible(d) ? n1 * r : 0.0f;
   r2 = divisible(d) ? n2 * r : 0.0f;
 }
@@ -267,7 +266,7 @@ __global__ void __launch_bounds__(kThreads, MINB) k_antidiff3v(Grid g, const flo
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
           const int i = c + 1;
-          const float rGb = NUG ? __fdividef(1.0f, 0.5f * (g0[i] + g0[i + 1])) : 1.0f;
+          const float rGb = NUG ? rcp(0.5f * (g0[i] + g0[i + 1])) : 1.0f;
           const float vqz = 0.25f * ((vz0[i] + vz0[i + 1]) + (vzm[i] + vzm[i + 1]));
           const float vqy = 0.25f * ((vy0[i] + vy0[i + 1]) + (vym[i] + vym[i + 1]));
           res[2][c] = face<IGA, TOT>(p00[i], p00[i + 1], p00[i - 1], p00[i + 2], rGb, vx[i],
@@ -289,7 +288,7 @@ __global__ void __launch_bounds__(kThreads, MINB) k_antidiff3v(Grid g, const flo
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
           const int i = c + 1;
-          const float rGb = NUG ? __fdividef(1.0f, 0.5f * (g0[i] + g1[i])) : 1.0f;
+          const float rGb = NUG ? rcp(0.5f * (g0[i] + g1[i])) : 1.0f;
           const float vqz = 0.25f * ((vz00[i] + vz01[i]) + (vzm0[i] + vzm1[i]));
           const float vqx = 0.25f * ((vx0[i] + vx1[i]) + (vx0[i - 1] + vx1[i - 1]));
           res[1][c] = face<IGA, TOT>(p00[i], p01[i], p0m[i], p02[i], rGb, vy[i],
@@ -312,7 +311,7 @@ __global__ void __launch_bounds__(kThreads, MINB) k_antidiff3v(Grid g, const flo
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
           const int i = c + 1;
-          const float rGb = NUG ? __fdividef(1.0f, 0.5f * (g0[i] + g1[i])) : 1.0f;
+          const float rGb = NUG ? rcp(0.5f * (g0[i] + g1[i])) : 1.0f;
           const float vqy = 0.25f * ((vy0[i] + vy1[i]) + (vy0m[i] + vy1m[i]));
           const float vqx = 0.25f * ((vx0[i] + vx1[i]) + (vx0[i - 1] + vx1[i - 1]));
           res[0][c] = face<IGA, TOT>(p00[i], p10[i], pm0[i], p20[i], rGb, vz[i],
@@ -355,7 +354,7 @@ constexpr int kCThreads = 32 * kCWarps;
 template <bool UNIT>
 __device__ __forceinline__ float fluxv(float L, float R, float V) {
   if constexpr (UNIT) return V;
-  else return posp(V) * L + negp(V) * R;
+  else return flux(L, R, V);
 }
 // ---------------------------------------------------------------- pass 1 and the FCT bounds
 // Pass 1 (Eqs. 4-5) and the FCT bounds (Sect. 3.1.4: extrema of psi^n and psi^(1) over the cell
@@ -381,12 +380,13 @@ template <bool KAHAN>
 __device__ __forceinline__ float donor1(float p, const float (&np)[3], const float (&nm)[3], const float (&vp)[3],
                                         const float (&vm)[3], float Gi, bool nug) {
   float s = p, comp = 0.0f;
+  const float rG = nug ? rcp(Gi) : 1.0f;  // one reciprocal serves the six terms
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const float Fp = fluxv<false>(p, np[d], vp[d]);
     const float Fm = fluxv<false>(nm[d], p, vm[d]);
-    const float t0 = nug ? -__fdividef(Fp, Gi) : -Fp;
-    const float t1 = nug ? __fdividef(Fm, Gi) : Fm;
+    const float t0 = nug ? -(Fp * rG) : -Fp;
+    const float t1 = nug ? Fm * rG : Fm;
     if constexpr (KAHAN) {
       float yk = t0 - comp;
       float u = s + yk;
@@ -545,17 +545,15 @@ __global__ void __launch_bounds__(kCThreads) k_p1b3v(Grid g, const float* __rest
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
         const int i = c + 1;
-        float h = a0[i] > b0[i] ? a0[i] : b0[i];
-        float l = a0[i] < b0[i] ? a0[i] : b0[i];
+        float h = maxv(a0[i], b0[i]);
+        float l = minv(a0[i], b0[i]);
         // neighbours in the order z-1, z+1, y-1, y+1, x-1, x+1; psi^n before psi^(1)
         const float ca[6] = {azm[c], azp[c], ad[c], au[c], a0[i - 1], a0[i + 1]};
         const float cb[6] = {bzm[c], bzp[c], bd[c], bu[c], b0[i - 1], b0[i + 1]};
 #pragma unroll
         for (int j = 0; j < 6; ++j) {
-          h = ca[j] > h ? ca[j] : h;
-          h = cb[j] > h ? cb[j] : h;
-          l = ca[j] < l ? ca[j] : l;
-          l = cb[j] < l ? cb[j] : l;
+          h = max3(h, ca[j], cb[j]);
+          l = min3(l, ca[j], cb[j]);
         }
         hi[c] = h;
         lo[c] = l;
@@ -623,37 +621,43 @@ __device__ __forceinline__ void factors1(float p, float pzp, float pzm, float py
                                          float vzp, float vzm, float vyp, float vym, float vxp, float vxm, float Gi,
                                          float mxi, float mni, float& bu, float& bd) {
   float in = 0.0f, ou = 0.0f;
+  // [x]+ = x - [x]- and [x]- = x - [x]+ are exact, so the outflow sum takes the inflow sum's
+  // extrema (adds instead of min/max on the half-rate pipe)
+  auto add = [&](float Fp, float Fm) {
+    const float n = negp(Fp), q = posp(Fm);
+    in = in + (q - n);
+    ou = ou + ((Fp - n) - (Fm - q));
+  };
   {
     const float Fp = fluxv<UNIT>(p, pzp, vzp), Fm = fluxv<UNIT>(pzm, p, vzm);
-    in = in + (posp(Fm) - negp(Fp));
-    ou = ou + (posp(Fp) - negp(Fm));
+    add(Fp, Fm);
   }
   {
     const float Fp = fluxv<UNIT>(p, pyp, vyp), Fm = fluxv<UNIT>(pym, p, vym);
-    in = in + (posp(Fm) - negp(Fp));
-    ou = ou + (posp(Fp) - negp(Fm));
+    add(Fp, Fm);
   }
   {
     const float Fp = fluxv<UNIT>(p, pxp, vxp), Fm = fluxv<UNIT>(pxm, p, vxm);
-    in = in + (posp(Fm) - negp(Fp));
-    ou = ou + (posp(Fp) - negp(Fm));
+    add(Fp, Fm);
   }
-  bu = in > 0.0f ? __fdividef(Gi * posp(mxi - p), in) : 1.0f;
-  bd = ou > 0.0f ? __fdividef(Gi * posp(p - mni), ou) : 1.0f;
+  // min(1, x / |s|): the limiter uses min(1, beta, beta); 1 for s = 0 (inf or NaN, which min ignores)
+  bu = min1(fdiv(Gi * posp(mxi - p), fabsf(in)));
+  bd = min1(fdiv(Gi * posp(p - mni), fabsf(ou)));
 }
 
-// The limited advector V min(1, a, b) of a face between L and R: the upwind side's outflow
-// factor and the downwind side's inflow factor (by the direction of the unlimited flux)
+// The limited advector h = V min(a, b) of a face between L and R, the factors (at most 1) being
+// the upwind side's outflow factor and the downwind side's inflow factor by the direction of the
+// unlimited flux, and the flux with it: h has V's sign or is 0, so both fluxes take the same
+// upwind value and one selection serves them
 template <bool UNIT>
-__device__ __forceinline__ float limited(float L, float R, float V, float buL, float bdL, float buR, float bdR) {
-  const float F = fluxv<UNIT>(L, R, V);
+__device__ __forceinline__ float limited(float L, float R, float V, float buL, float bdL, float buR, float bdR,
+                                         float& Fh) {
+  const float up = UNIT ? 1.0f : (V > 0.0f ? L : R);
+  const float F = UNIT ? V : V * up;
   const bool right = F > 0.0f || (F == 0.0f && V > 0.0f);
-  const float a = right ? bdL : buL;
-  const float b = right ? buR : bdR;
-  float m = 1.0f;
-  m = minv(a, m);
-  m = minv(b, m);
-  return V * m;
+  const float h = V * minv(right ? bdL : buL, right ? buR : bdR);
+  Fh = UNIT ? h : h * up;
+  return h;
 }
 
 template <int NC, bool NUG, bool UNIT, bool LIM>
@@ -801,13 +805,13 @@ __global__ void __launch_bounds__(kCThreads, 2) k_corr3v(Grid g, const float* __
         center<NC>(Q0 + (w + 1) * W, lane, p);
         center<NC>(UQ + w * W, lane, bu);
         center<NC>(DQ + w * W, lane, bd);
-        float Gc[NC];  // G of the cells (the divisor of the donor terms)
+        float rGc[NC];  // 1/G of the cells
 #pragma unroll
-        for (int c = 0; c < NC; ++c) { acc[c] = p[c]; Gc[c] = NUG ? g_m[c] : 1.0f; }
+        for (int c = 0; c < NC; ++c) { acc[c] = p[c]; rGc[c] = NUG ? rcp(g_m[c]) : 1.0f; }
         // the donor terms of one dimension: -F+/G then +F-/G, added in that order
         auto donor_d = [&](int c, float Fp, float Fm) {
-          const float t0 = NUG ? -__fdividef(Fp, Gc[c]) : -Fp;
-          const float t1 = NUG ? __fdividef(Fm, Gc[c]) : Fm;
+          const float t0 = NUG ? -(Fp * rGc[c]) : -Fp;
+          const float t1 = NUG ? Fm * rGc[c] : Fm;
           acc[c] = acc[c] + t0;
           acc[c] = acc[c] + t1;
         };
@@ -821,9 +825,10 @@ __global__ void __launch_bounds__(kCThreads, 2) k_corr3v(Grid g, const float* __
           center<NC>(DQm + w * W, lane, dzm);
 #pragma unroll
           for (int c = 0; c < NC; ++c) {
-            const float hp = limited<UNIT>(p[c], nzp[c], vz_m[c], bu[c], bd[c], uzp[c], dzp[c]);
-            const float hm = limited<UNIT>(nzm[c], p[c], vz_mm[c], uzm[c], dzm[c], bu[c], bd[c]);
-            donor_d(c, fluxv<UNIT>(p[c], nzp[c], hp), fluxv<UNIT>(nzm[c], p[c], hm));
+            float Fp, Fm;
+            const float hp = limited<UNIT>(p[c], nzp[c], vz_m[c], bu[c], bd[c], uzp[c], dzp[c], Fp);
+            limited<UNIT>(nzm[c], p[c], vz_mm[c], uzm[c], dzm[c], bu[c], bd[c], Fm);
+            donor_d(c, Fp, Fm);
             hz[c] = hp;
           }
         }
@@ -839,9 +844,10 @@ __global__ void __launch_bounds__(kCThreads, 2) k_corr3v(Grid g, const float* __
           center<NC>(DQ + (w - 1) * W, lane, dd);
 #pragma unroll
           for (int c = 0; c < NC; ++c) {
-            const float hp = limited<UNIT>(p[c], nyp[c], vy[c], bu[c], bd[c], uu[c], du[c]);
-            const float hm = limited<UNIT>(nym[c], p[c], vym[c], ud[c], dd[c], bu[c], bd[c]);
-            donor_d(c, fluxv<UNIT>(p[c], nyp[c], hp), fluxv<UNIT>(nym[c], p[c], hm));
+            float Fp, Fm;
+            const float hp = limited<UNIT>(p[c], nyp[c], vy[c], bu[c], bd[c], uu[c], du[c], Fp);
+            limited<UNIT>(nym[c], p[c], vym[c], ud[c], dd[c], bu[c], bd[c], Fm);
+            donor_d(c, Fp, Fm);
             hy[c] = hp;
           }
         }
@@ -854,9 +860,10 @@ __global__ void __launch_bounds__(kCThreads, 2) k_corr3v(Grid g, const float* __
 #pragma unroll
           for (int c = 0; c < NC; ++c) {
             const int i = c + 1;
-            const float hp = limited<UNIT>(p[c], pc[i + 1], vx[i], bu[c], bd[c], uc[i + 1], dc[i + 1]);
-            const float hm = limited<UNIT>(pc[i - 1], p[c], vx[i - 1], uc[i - 1], dc[i - 1], bu[c], bd[c]);
-            donor_d(c, fluxv<UNIT>(p[c], pc[i + 1], hp), fluxv<UNIT>(pc[i - 1], p[c], hm));
+            float Fp, Fm;
+            const float hp = limited<UNIT>(p[c], pc[i + 1], vx[i], bu[c], bd[c], uc[i + 1], dc[i + 1], Fp);
+            limited<UNIT>(pc[i - 1], p[c], vx[i - 1], uc[i - 1], dc[i - 1], bu[c], bd[c], Fm);
+            donor_d(c, Fp, Fm);
             hx[c] = hp;
           }
         }
