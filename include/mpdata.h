@@ -33,8 +33,9 @@
  * process or throws (the C analogue of the library's std::runtime_error,
  * Sect. 2.4).  All device work is enqueued on the handle's stream and is
  * asynchronous; a device-side failure is reported by the next call on the
- * handle that synchronises (mpdata_reduce, mpdata_sync).  No kernel of this
- * library waits on another block of its grid (block barriers only); the reverse
+ * handle that synchronises (mpdata_reduce, mpdata_sync).  The blocks of a grid
+ * wait for each other only inside one thread-block cluster, whose blocks the
+ * hardware runs at the same time (the 1D path's cluster barrier); the reverse
  * step's kernels, launched as programmatic dependents, wait only for the
  * completion of the kernel before them on the stream.  No call can hang on a
  * device-side wait.
@@ -152,9 +153,9 @@ int mpdata_sw_reset(mpdata_t h);
 
 /*
  * Advances psi in place by n_steps >= 1 steps (the paper's advance(), Sect. 3.2.5).
- * 2D steps with n_iters = 2 run fused kernels (one launch per step), 1D fields of up
- * to 2235 (FP64) / 4470 (FP32) cells run the whole call in one launch, the rest run
- * one kernel per sub-step.
+ * 2D steps with n_iters = 2 run fused kernels (one launch per step), 1D fields short enough for
+ * one thread-block cluster (about 10000 cells with two passes) run the whole call in one launch,
+ * and so do such 1D systems with trapezoidal sources; the rest run one kernel per sub-step.
  * gc (host array of ndims device pointers): advector components, constant over
  * the call.  g: G field (required iff MPDATA_NUG, else NULL).  r: source term R
  * (required iff an RHS bit is set, else NULL), dt its time step.
@@ -281,9 +282,9 @@ int mpdata_check_courant(mpdata_t h, const void* const* gc, const void* g, doubl
 /*
  * Asks the handle to stop: later mpdata_step / mpdata_advance calls return
  * MPDATA_ESTOPPED without enqueuing work, and a multi-step call stops after the
- * step in progress (the paper's panic flag, Sect. 3.2.5).  A 1D field small
- * enough for shared memory runs every step of a call in one launch; for it the
- * request takes effect at the next call.  Thread-safe.  mpdata_clear_stop
+ * step in progress (the paper's panic flag, Sect. 3.2.5).  A 1D field (or 1D system with
+ * trapezoidal sources) short enough for one cluster runs every step of a call in one launch; for
+ * it the request takes effect at the next call.  Thread-safe.  mpdata_clear_stop
  * re-arms the handle.
  */
 int mpdata_request_stop(mpdata_t h);

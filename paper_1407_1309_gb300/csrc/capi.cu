@@ -72,13 +72,20 @@ int run_trapez(mpdata_s* h, const T* psi_in, T* psi_out, const void* const* gcv,
   if (!h->rhs_lin) return MPDATA_EINVAL;
   mpd::TrapezMat m;
   if (!mpd::trapez_matrix(m, h->rhs_A.data(), h->n_fields, dt)) return MPDATA_EINVAL;
+  const long long n = h->grids[0].N;
+  const T* b = static_cast<const T*>(h->rhs_b);
+  // a 1D system short enough for one cluster: every step of the call in one launch
+  if (h->nd == 1 && !(h->opts & MPDATA_STAGED) && !gc_scale) {
+    const int rc = mpd::line1d_steps<T>(h->grids[0], mpd::make_opts(h->opts, h->n_iters), psi_in, psi_out,
+                                        static_cast<const T*>(gcv[0]), g, nullptr, static_cast<T>(dt), n_steps, &m, b,
+                                        h->stream);
+    if (rc != MPDATA_EUNSUPPORTED) return rc;
+  }
   if (!h->trapez_buf && cudaMalloc(&h->trapez_buf, static_cast<size_t>(h->total) * sizeof(T)) != cudaSuccess) {
     h->trapez_buf = nullptr;
     return MPDATA_ENOMEM;
   }
-  const long long n = h->grids[0].N;
   T* S = static_cast<T*>(h->trapez_buf);
-  const T* b = static_cast<const T*>(h->rhs_b);
   for (int s = 0; s < n_steps; ++s) {
     if (h->stop.load(std::memory_order_relaxed)) return MPDATA_ESTOPPED;
     if (mpd::trapez_pre<T>(m, n, static_cast<T>(dt), s == 0 ? psi_in : psi_out, b, S, h->stream) != cudaSuccess)
@@ -103,11 +110,14 @@ int run_advance(mpdata_s* h, const T* psi_in, T* psi_out, const void* const* gcv
   // Every step reads one buffer and writes another: the result alternates between
   // psi_out and the handle's ping-pong buffer so that the last step lands in psi_out.
   // In place with an odd step count, psi is first copied to the ping-pong buffer.
-  // a small 1D field runs every step of the call in one launch of one block (it reads the
-  // whole field before writing, so in place needs no copy)
+  // a 1D field runs every step of the call in one launch: of one cluster, or, where a step reaches
+  // too many cells for that (many passes), of one block.  Both read the whole field before
+  // writing, so in place needs no copy
   if (h->nd == 1 && h->n_fields == 1 && !o.staged && !gc_scale) {
-    const int rc = mpd::steps1d<T>(h->grids[0], o, psi_in, psi_out, gc[0], g, r, static_cast<T>(dt), n_steps,
-                                   h->stream);
+    int rc = mpd::line1d_steps<T>(h->grids[0], o, psi_in, psi_out, gc[0], g, r, static_cast<T>(dt), n_steps, nullptr,
+                                  nullptr, h->stream);
+    if (rc == MPDATA_EUNSUPPORTED)
+      rc = mpd::steps1d<T>(h->grids[0], o, psi_in, psi_out, gc[0], g, r, static_cast<T>(dt), n_steps, h->stream);
     if (rc != MPDATA_EUNSUPPORTED) return rc;
   }
   T* X = psi_out;

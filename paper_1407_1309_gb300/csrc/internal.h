@@ -153,6 +153,27 @@ template <typename T>
 int steps1d(const Grid& g, const Opts& o, const T* psi_in, T* psi_out, const T* gc, const T* G, const T* R, T dt,
             int n_steps, cudaStream_t st);
 
+// Trapezoidal source scheme (rhs.cu) for a system of E <= kTrapezMax equations of n cells each,
+// stored field after field: pre writes psi + dt/2 (A psi + b) into out; post turns the advected
+// fields into psi^{n+1} = Minv (psi* + dt/2 b) in place, Minv = (I - dt/2 A)^{-1}.
+constexpr int kTrapezMax = 8;
+struct TrapezMat {
+  int E;
+  double A[kTrapezMax * kTrapezMax];
+  double Minv[kTrapezMax * kTrapezMax];
+};
+// Minv of I - dt/2 A by Gauss-Jordan elimination with partial pivoting; false if singular.
+bool trapez_matrix(TrapezMat& m, const double* A, int E, double dt);
+
+// Every step of a call for a 1D field, or (m not null: its matrices and b) for a system of m->E 1D
+// equations of g.N cells each with trapezoidal sources, in one launch of one thread-block cluster
+// (line1d.cu): the field in registers, halos exchanged through distributed shared memory.
+// MPDATA_EUNSUPPORTED (nothing launched) for the divergent-flow term, open edges, steps that reach
+// more than 12 cells and fields too long for one cluster.
+template <typename T>
+int line1d_steps(const Grid& g, const Opts& o, const T* psi_in, T* psi_out, const T* gc, const T* G, const T* R, T dt,
+                 int n_steps, const TrapezMat* m, const T* b, cudaStream_t st);
+
 // Intermediates of one forward step kept for the adjoint (n_iters <= kTapeMax).
 constexpr int kTapeMax = 4;
 template <typename T>
@@ -173,17 +194,6 @@ template <typename T>
 cudaError_t staged_forward_tape(const Grid& g, const Opts& o, const T* const* gc, const T* G,
                                 const Tape<T>& tp, T* const* psi_out_levels, T* psi_next, cudaStream_t st);
 
-// Trapezoidal source scheme (rhs.cu) for a system of E <= kTrapezMax equations of n cells each,
-// stored field after field: pre writes psi + dt/2 (A psi + b) into out; post turns the advected
-// fields into psi^{n+1} = Minv (psi* + dt/2 b) in place, Minv = (I - dt/2 A)^{-1}.
-constexpr int kTrapezMax = 8;
-struct TrapezMat {
-  int E;
-  double A[kTrapezMax * kTrapezMax];
-  double Minv[kTrapezMax * kTrapezMax];
-};
-// Minv of I - dt/2 A by Gauss-Jordan elimination with partial pivoting; false if singular.
-bool trapez_matrix(TrapezMat& m, const double* A, int E, double dt);
 template <typename T>
 cudaError_t trapez_pre(const TrapezMat& m, long long n, T dt, const T* psi, const T* b, T* out, cudaStream_t st);
 template <typename T>
