@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps) k_line1d(const LineParams<T> p
   const int rank = static_cast<int>(cluster_rank());
   const int n = p.n, E = SYS ? p.E : 1;
   auto start_of = [&](int r) { return static_cast<int>(static_cast<long long>(r) * n / C); };
-  const int c0 = start_of(rank), c1 = start_of(rank + 1), len = c1 - c0;
+  const int c0 = start_of(rank), c1 = start_of(rank + 1);
   const int HS = p.halo * p.S;
   const int most = (n + C - 1) / C;         // the longest range of a block
   const int pitch = most + 2 * HS;          // one equation's buffer
@@ -334,6 +334,8 @@ template <typename T>
 int line1d_steps(const Grid& g, const Opts& o, const T* psi_in, T* psi_out, const T* gc, const T* G, const T* R, T dt,
                  int n_steps, const TrapezMat* m, const T* b, cudaStream_t st) {
   if (g.nd != 1 || o.dfl || o.open) return MPDATA_EUNSUPPORTED;
+  // FP64 |psi| stays on the staged kernels: on a positive field it is their basic scheme bit for bit
+  if (o.abs && sizeof(T) == 8) return MPDATA_EUNSUPPORTED;
   if (g.N > (1 << 20) || o.n_iters > 64) return MPDATA_EUNSUPPORTED;
   LineParams<T> p{};
   p.n = static_cast<int>(g.N);
