@@ -56,6 +56,11 @@ int band_tape(const Grid& g, const Opts& o, const StepArgs<T>& a, T* tape, cudaS
 int fused_step_comp(const Grid& g, const Opts& o, const StepArgs<float>& a, const float* lo_in, float* lo_out,
                     cudaStream_t st);
 
+// The fused 2D step of an FP32 field with the variable-sign option, the divergent-flow term or both
+// (fused2d_ext.cu, warp march); MPDATA_EUNSUPPORTED with Kahan summation.  FP64 fields with these
+// options stay on the staged kernels.
+int fused_step_ext(const Grid& g, const Opts& o, const StepArgs<float>& a, cudaStream_t st);
+
 // The same step with one marching front per block of warps (band2d.cu).
 template <typename T>
 int band_step(const Grid& g, const Opts& o, const StepArgs<T>& a, cudaStream_t st);
