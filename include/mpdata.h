@@ -67,12 +67,11 @@ enum {
   MPDATA_STAGED = 128u,     /* run the one-kernel-per-sub-step path even where a fused
                                kernel covers the case (comparison and testing) */
   MPDATA_ABS = 256u,        /* variable-sign fields: |psi| in every psi-fraction of the
-                               pseudo-velocity (Sect. 3.1.5); excludes MPDATA_IGA.  Runs on
-                               the one-kernel-per-sub-step path; no reverse step */
+                               pseudo-velocity (Sect. 3.1.5); excludes MPDATA_IGA */
   MPDATA_DFL = 512u,        /* divergent flow (Sect. 3.1.3): the pseudo-velocity gains
                                -1/4 V (div_i + div_{i+e_d}) / Gb, div_j the advector's
                                difference summed over the dimensions across cell j; excludes
-                               MPDATA_IGA.  One-kernel-per-sub-step path; no reverse step */
+                               MPDATA_IGA */
   /* Open edges (Sect. 2.4, bcond::open: a zero-divergence condition on the domain edges)
      along dimension d, bit MPDATA_OPEN0 << d; both ends of that dimension, the others stay
      periodic.  The halo cells beyond an open edge hold the edge cell's value; the n-1 faces
@@ -80,7 +79,7 @@ enum {
      one shorter than the field along its own dimension, Sect. 3.2.5: entry n-1 is not read),
      and each of the two boundary faces carries, for the advector and every pass's
      pseudo-velocity, the value of the adjacent interior face.  An open dimension needs n >= 2.
-     One-kernel-per-sub-step path; no reverse step (MPDATA_EUNSUPPORTED) */
+     No reverse step (MPDATA_EUNSUPPORTED) */
   MPDATA_OPEN0 = 1024u,
   MPDATA_OPEN1 = 2048u,
   MPDATA_OPEN2 = 4096u,
@@ -153,7 +152,8 @@ int mpdata_sw_reset(mpdata_t h);
 
 /*
  * Advances psi in place by n_steps >= 1 steps (the paper's advance(), Sect. 3.2.5).
- * 2D steps with n_iters = 2 run fused kernels (one launch per step), 1D fields short enough for
+ * 2D steps run fused kernels (one launch per step; more than two passes, the third-order terms and
+ * open edges as a shared-memory tile kernel), 1D fields short enough for
  * one thread-block cluster (about 10000 cells with two passes) run the whole call in one launch,
  * and so do such 1D systems with trapezoidal sources; the rest run one kernel per sub-step.
  * gc (host array of ndims device pointers): advector components, constant over

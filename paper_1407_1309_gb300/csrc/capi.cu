@@ -173,6 +173,7 @@ int run_advance(mpdata_s* h, const T* psi_in, T* psi_out, const void* const* gcv
       a.dt = static_cast<T>(dt);
       a.gc_scale = scale;
       int rc = o.staged ? MPDATA_EUNSUPPORTED : mpd::fused_step<T>(gr, o, a, nullptr, h->stream);
+      if (rc == MPDATA_EUNSUPPORTED && !o.staged) rc = mpd::tile2d_step<T>(gr, o, a, 1, 0, h->stream);
       if (rc == MPDATA_EUNSUPPORTED) rc = cuda_status(mpd::staged_step<T>(gr, o, a, ss, h->stream));
       if (rc != MPDATA_OK) return rc;
     }
@@ -283,6 +284,8 @@ int run_sw(mpdata_s* h, T* state, double dt, double dx, double eps, int n_steps)
     h->sw_first = false;
     if (mpd::sw_force<T>(gr, cur, static_cast<T>(0.5 * dt), static_cast<T>(dx), h->stream) != cudaSuccess)
       return MPDATA_ECUDA;
+    // every field by the fused march where that covers the options, else all fields in one launch
+    // of the tile kernel (2D), else field by field on the staged kernels
     for (int f = 0; f <= nd; ++f) {
       mpd::StepArgs<T> a;
       a.psi_in = cur + static_cast<long long>(f) * n;
@@ -293,6 +296,10 @@ int run_sw(mpdata_s* h, T* state, double dt, double dx, double eps, int n_steps)
       a.dt = static_cast<T>(dt);
       a.gc_scale = T(1);
       int rc = o.staged ? MPDATA_EUNSUPPORTED : mpd::fused_step<T>(gr, o, a, nullptr, h->stream);
+      if (rc == MPDATA_EUNSUPPORTED && !o.staged && f == 0) {
+        rc = mpd::tile2d_step<T>(gr, o, a, nd + 1, n, h->stream);
+        if (rc == MPDATA_OK) break;
+      }
       if (rc == MPDATA_EUNSUPPORTED) rc = cuda_status(mpd::staged_step<T>(gr, o, a, ss, h->stream));
       if (rc != MPDATA_OK) return rc;
     }

@@ -61,6 +61,13 @@ int fused_step_comp(const Grid& g, const Opts& o, const StepArgs<float>& a, cons
 // options stay on the staged kernels.
 int fused_step_ext(const Grid& g, const Opts& o, const StepArgs<float>& a, cudaStream_t st);
 
+// One out-of-place step of `fields` 2D fields of one shape as a shared-memory tile kernel
+// (tile2d.cu): any options, passes and open edges whose reach fits.  psi and out of field f start
+// f * `field` elements behind a.psi_in and a.psi_out; the advector, G and R are shared.
+// MPDATA_EUNSUPPORTED (nothing launched) for one pass, in place, or a reach too large.
+template <typename T>
+int tile2d_step(const Grid& g, const Opts& o, const StepArgs<T>& a, int fields, long long field, cudaStream_t st);
+
 // The same step with one marching front per block of warps (band2d.cu).
 template <typename T>
 int band_step(const Grid& g, const Opts& o, const StepArgs<T>& a, cudaStream_t st);
