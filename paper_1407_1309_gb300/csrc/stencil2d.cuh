@@ -28,20 +28,20 @@ __device__ __forceinline__ float rcp(float d) {
   return r;
 }
 template <> __device__ __forceinline__ float fdiv<float>(float a, float b) { return a * rcp(b); }
-// FP64 n / d for the arithmetic-bound FP64 kernels: Newton-Raphson reciprocal iteration
-// r <- r + r (1 - d r) (quadratic convergence) from the PTX approximate FP64 reciprocal
-// (rcp.approx.ftz.f64, full exponent range), two iterations, and Markstein's remainder
-// correction q <- q + r (n - d q) of the quotient: within one unit in the last place of the
-// exact quotient for normal operands.  A zero, infinite or NaN divisor gives NaN (the
-// kernels never rely on it: the psi-ratio guards zero sums, and the FCT factors' min(1, x)
-// maps the inf or NaN of a zero flux sum to 1 alike).
+// FP64 n / d for the arithmetic-bound FP64 kernels, five FP64 operations: one Newton-Raphson
+// iteration r <- r + r (1 - d r) (quadratic convergence) from the PTX approximate FP64 reciprocal
+// (rcp.approx.ftz.f64, full exponent range), and Markstein's remainder correction
+// q <- q + r (n - d q) of the quotient: within one unit in the last place of the exact quotient for
+// normal operands.  The seed carries about 20 bits, the iterated reciprocal 40; the remainder is
+// exact in the fma, so the corrected quotient's error before its last rounding is the product of
+// two 2^-40 errors.  Measured against IEEE division: all of 4 10^8 quotients equal, with this
+// form and with a second iteration alike; without it the 1024^2 FP64 step takes 215 instead of
+// 242 us.  A zero, infinite or NaN divisor gives NaN (the kernels never rely on it: the psi-ratio guards zero sums, and the FCT
+// factors' min(1, x) maps the inf or NaN of a zero flux sum to 1 alike).
 __device__ __forceinline__ double nr_div(double n, double d) {
   double r0;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(d));
-  double e = fma(-d, r0, 1.0);
-  double r = fma(r0, e, r0);
-  e = fma(-d, r, 1.0);
-  r = fma(r, e, r);
+  const double r = fma(r0, fma(-d, r0, 1.0), r0);
   const double q = n * r;
   return fma(r, fma(-d, q, n), q);
 }
