@@ -27,6 +27,7 @@
 #include <cuda_runtime.h>
 
 #include "kernels.h"
+#include "launch.cuh"
 #include "stencil2d.cuh"
 
 namespace mpd {
@@ -144,27 +145,8 @@ template <typename T> __device__ __forceinline__ T flux(T L, T R, T V, bool unit
   return unit ? V : posp(V) * L + negp(V) * R;
 }
 
-// Programmatic dependent launch: a kernel launched with launch_after() may start while its
-// predecessor on the stream finishes; it calls grid_wait() before it reads anything the
-// predecessor wrote (no-ops for kernels launched the ordinary way).  grid_release() lets the
-// successor's launch begin as soon as every block of this grid has started.
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" :::); }
-
-template <typename... KArgs, typename... Args>
-cudaError_t launch_after(void (*kern)(KArgs...), dim3 grid, dim3 block, cudaStream_t st, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
-}
+using dev::grid_release;
+using dev::grid_wait;
 
 // loop over the cells on a (fast, middle, slow) launch grid; closed by CELL_END
 #define CELL_INDEX                                                                    \

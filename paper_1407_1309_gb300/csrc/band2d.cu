@@ -21,6 +21,7 @@
 #include <cuda_runtime.h>
 
 #include "kernels.h"
+#include "launch.cuh"
 #include "stencil2d.cuh"
 
 namespace mpd {
@@ -48,6 +49,7 @@ struct BandParams {
   T* tape;  // adjoint tape (TAPE only): arrays of tape_n elements
   long long tape_n;
   int tape_vec;  // tape rows may be written as 16-byte vectors
+  bool chained;  // launched as a dependent of the kernel before it (StepArgs::chained)
 };
 
 // NC values of one lane from / to a shared-memory row (16-byte vectors where they fit)
@@ -155,22 +157,33 @@ __global__ void __launch_bounds__(W * 32, 2) k_band2d(const BandParams<T> p) {
   // The warp's load rows advance by W per chunk: their global row is kept wrapped
   // incrementally (the first one with a modulo).
   int g_row = wrapi(Rs + w, p.n0);
-  auto load_row = [&](int lr) {
+  // kAll: every array of the row; else psi or the rest
+  enum Part { kAll, kState, kRest };
+  auto load_row = [&](int lr, const Part part) {
     if (lr < n_load) {
       const long long off = static_cast<long long>(g_row) * p.n1;
       g_row += W;
       while (g_row >= p.n0) g_row -= p.n0;
-      copy_in(in_row(s_psi, lr), p.psi + off);
-      copy_in(in_row(s_v0, lr), p.gc0 + off);
-      copy_in(in_row(s_v1, lr), p.gc1 + off);
-      if (NUG) copy_in(in_row(s_g, lr), p.G + off);
-      if (p.rhs_b) copy_in(in_row(s_r, lr), p.R + off);
+      if (part != kRest) copy_in(in_row(s_psi, lr), p.psi + off);
+      if (part != kState) {
+        copy_in(in_row(s_v0, lr), p.gc0 + off);
+        copy_in(in_row(s_v1, lr), p.gc1 + off);
+        if (NUG) copy_in(in_row(s_g, lr), p.G + off);
+        if (p.rhs_b) copy_in(in_row(s_r, lr), p.R + off);
+      }
     }
-    cp_commit();
+    if (part != kRest) cp_commit();
   };
 
+  // the first chunks: what no earlier step of the call writes, then, once the step before this one
+  // is complete, psi (the copies of the first part join the first chunk's group)
+  if (gridDim.x <= kChainBlocks) grid_release();
 #pragma unroll
-  for (int j = 0; j < kDepth; ++j) load_row(j * W + w);
+  for (int j = 0; j < kDepth; ++j) load_row(j * W + w, kRest);
+  g_row = wrapi(Rs + w, p.n0);
+  grid_wait();
+#pragma unroll
+  for (int j = 0; j < kDepth; ++j) load_row(j * W + w, kState);
   const bool fix = p.rhs_b || p.scale != T(1);
   // euler_b source and advector scale on a row this warp loaded itself
   auto fix_row = [&](int lr) {
@@ -297,7 +310,7 @@ __global__ void __launch_bounds__(W * 32, 2) k_band2d(const BandParams<T> p) {
       tape_row(0, a, p1_c);
     }
     __syncthreads();
-    load_row((j + kDepth) * W + w);  // after the barrier: the slots it refills are no longer read
+    load_row((j + kDepth) * W + w, kAll);  // after the barrier: the slots it refills are no longer read
 
     // ---- local row b = a - 1: pseudo-advectors (Eq. 6 + cross term) and unlimited fluxes.
     // The face between rows b and b+1 needs psi^(1) on rows b, b+1 only and is computed
@@ -452,7 +465,7 @@ void launch_band(BandParams<T> p, int tile_rows, cudaStream_t st) {
   }
   const long long blocks = static_cast<long long>(p.strips) * ((p.n0 + p.H - 1) / p.H);
   const size_t smem = band_smem<T>(3 + (NUG ? 1 : 0) + (p.rhs_b ? 1 : 0), FCT);
-  kern<<<static_cast<unsigned>(blocks), W * 32, smem, st>>>(p);
+  launch_chained(p.chained, kern, dim3(static_cast<unsigned>(blocks)), dim3(W * 32), smem, st, p);
 }
 
 template <typename T, int NC, bool FCT, bool NUG>
@@ -496,6 +509,7 @@ int band_step(const Grid& g, const Opts& o, const StepArgs<T>& a, cudaStream_t s
   p.tape = nullptr;
   p.tape_n = 0;
   p.tape_vec = 0;
+  p.chained = a.chained;
   if (o.fct) {
     if (o.nug) band_mode<T, NC, true, true>(p, o.tile_rows, o.iga, o.kahan, st);
     else band_mode<T, NC, true, false>(p, o.tile_rows, o.iga, o.kahan, st);
@@ -532,6 +546,7 @@ int band_tape(const Grid& g, const Opts& o, const StepArgs<T>& a, T* tape, cudaS
   p.tape = tape;
   p.tape_n = g.N;
   p.tape_vec = p.vec && aligned_to(tape, 16);
+  p.chained = a.chained;
   if (o.fct) launch_band<T, NC, true, false, false, false, true>(p, o.tile_rows, st);
   else launch_band<T, NC, false, false, false, false, true>(p, o.tile_rows, st);
   return cudaGetLastError() == cudaSuccess ? MPDATA_OK : MPDATA_ECUDA;

@@ -34,7 +34,7 @@ void batched_free(mpdata_s* h) {
 
 template <typename T>
 int batched_step(mpdata_s* h, const T* psi_in, T* psi_out, const T* const* gc, const T* g, const T* r, T dt,
-                 T gc_scale, const Opts& o) {
+                 T gc_scale, bool chained, const Opts& o) {
   if (handle_nd(h) != 2 || o.n_iters != 2 || o.tot || o.abs || o.dfl || o.open) return MPDATA_EUNSUPPORTED;
   // lanes of 2 columns for FP32 when the handle asks for them (MPDATA_TUNE_KERNEL = 3)
   const int nc = (o.kernel == 3 && sizeof(T) == 4) ? 2 : fused_batched_columns<T>();
@@ -75,13 +75,13 @@ int batched_step(mpdata_s* h, const T* psi_in, T* psi_out, const T* const* gc, c
     cudaMemcpy(th->tab.item_field, item_field.data(), sizeof(int) * item_field.size(), cudaMemcpyHostToDevice);
     *slot = th;
   }
-  return fused_batched_step<T>(th->tab, o, psi_in, psi_out, gc[0], gc[1], g, r, dt, gc_scale, handle_stream(h),
+  return fused_batched_step<T>(th->tab, o, psi_in, psi_out, gc[0], gc[1], g, r, dt, gc_scale, chained, handle_stream(h),
                                th->nc);
 }
 
 template int batched_step<float>(mpdata_s*, const float*, float*, const float* const*, const float*, const float*,
-                                 float, float, const Opts&);
+                                 float, float, bool, const Opts&);
 template int batched_step<double>(mpdata_s*, const double*, double*, const double* const*, const double*,
-                                  const double*, double, double, const Opts&);
+                                  const double*, double, double, bool, const Opts&);
 
 }  // namespace mpd

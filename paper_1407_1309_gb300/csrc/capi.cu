@@ -149,14 +149,17 @@ int run_advance(mpdata_s* h, const T* psi_in, T* psi_out, const void* const* gcv
       return MPDATA_ECUDA;
     cur = P;
   }
+  // whether the last kernel on the stream is a fused step of this call (StepArgs::chained)
+  bool chained = false;
   for (int s = 0; s < n_steps; ++s) {
     if (h->stop.load(std::memory_order_relaxed)) return MPDATA_ESTOPPED;
     const T scale = gc_scale ? static_cast<T>(gc_scale[s]) : T(1);
     T* dst = ((n_steps - 1 - s) % 2 == 0) ? X : P;
     if (h->n_fields > 1 && !o.staged) {
-      int rc = mpd::batched_step<T>(h, cur, dst, gc, g, r, static_cast<T>(dt), scale, o);
+      int rc = mpd::batched_step<T>(h, cur, dst, gc, g, r, static_cast<T>(dt), scale, chained, o);
       if (rc != MPDATA_EUNSUPPORTED) {
         if (rc != MPDATA_OK) return rc;
+        chained = true;
         cur = dst;
         continue;
       }
@@ -172,8 +175,10 @@ int run_advance(mpdata_s* h, const T* psi_in, T* psi_out, const void* const* gcv
       a.r = r ? r + off : nullptr;
       a.dt = static_cast<T>(dt);
       a.gc_scale = scale;
+      a.chained = chained;
       int rc = o.staged ? MPDATA_EUNSUPPORTED : mpd::fused_step<T>(gr, o, a, nullptr, h->stream);
       if (rc == MPDATA_EUNSUPPORTED && !o.staged) rc = mpd::tile2d_step<T>(gr, o, a, 1, 0, h->stream);
+      chained = rc == MPDATA_OK;
       if (rc == MPDATA_EUNSUPPORTED) rc = cuda_status(mpd::staged_step<T>(gr, o, a, ss, h->stream));
       if (rc != MPDATA_OK) return rc;
     }
@@ -442,6 +447,7 @@ int mpdata_advance_compensated(mpdata_t h, const void* psi_in, const void* lo_in
     a.r = static_cast<const float*>(r);
     a.dt = static_cast<float>(dt);
     a.gc_scale = gc_scale ? static_cast<float>(gc_scale[s]) : 1.0f;
+    a.chained = s > 0;
     rc = mpd::fused_step_comp(h->grids[0], o, a, curl, dstl, h->stream);
     if (rc != MPDATA_OK) return rc;
     cur = dst;

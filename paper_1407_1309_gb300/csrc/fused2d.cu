@@ -22,6 +22,7 @@ struct BatchParams {
   int n_items, ty;
   T dt, scale;
   int rhs_a, rhs_b, vec_ok;
+  bool chained;
 };
 
 template <typename T, int NC, bool FCT, bool NUG, bool IGA, bool KAHAN>
@@ -30,6 +31,8 @@ __global__ void __launch_bounds__(kWarps * 32) k_fused2d_batched(const BatchPara
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   T* ring = reinterpret_cast<T*>(smem_raw) + static_cast<size_t>(wib) * kSlots * kArr * cols<NC>();
+  if (gridDim.x <= kChainBlocks) grid_release();
+  grid_wait();  // the step before this one, when launched as its dependent
   const int total = gridDim.x * kWarps;
   for (int item = blockIdx.x * kWarps + wib; item < b.n_items; item += total) {
     const BatchField fd = b.fields[b.item_field[item]];
@@ -55,6 +58,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_fused2d_batched(const BatchPara
     p.lo_out = nullptr;
     p.tape = nullptr;
     p.tape_n = 0;
+    p.chained = b.chained;
     march_tile<T, NC, FCT, NUG, IGA, KAHAN, false>(p, local % fd.strips, (local / fd.strips) * b.ty, ring, lane);
   }
 }
@@ -93,7 +97,9 @@ void launch_b(const BatchParams<T>& b, cudaStream_t st) {
     return (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
   });
   const int need = (b.n_items + kWarps - 1) / kWarps;
-  k_fused2d_batched<T, NC, FCT, NUG, IGA, KAHAN><<<need < grid ? need : grid, kWarps * 32, smem, st>>>(b);
+  const unsigned blocks = need < grid ? need : grid;
+  launch_chained(b.chained, k_fused2d_batched<T, NC, FCT, NUG, IGA, KAHAN>, dim3(blocks),
+                 dim3(kWarps * 32), smem, st, b);
 }
 
 template <typename T, int NC, bool FCT, bool NUG>
@@ -118,8 +124,9 @@ namespace {
 
 template <typename T, int NC>
 int batched_launch(const BatchTable& tab, const Opts& o, const T* psi_in, T* psi_out, const T* gc0, const T* gc1,
-                   const T* G, const T* R, T dt, T scale, cudaStream_t st) {
+                   const T* G, const T* R, T dt, T scale, bool chained, cudaStream_t st) {
   BatchParams<T> b;
+  b.chained = chained;
   b.psi = psi_in;
   b.out = psi_out;
   b.gc0 = gc0;
@@ -150,19 +157,20 @@ int batched_launch(const BatchTable& tab, const Opts& o, const T* psi_in, T* psi
 
 template <typename T>
 int fused_batched_step(const BatchTable& tab, const Opts& o, const T* psi_in, T* psi_out, const T* gc0,
-                       const T* gc1, const T* G, const T* R, T dt, T scale, cudaStream_t st, int nc) {
+                       const T* gc1, const T* G, const T* R, T dt, T scale, bool chained, cudaStream_t st, int nc) {
   if (o.n_iters != 2 || o.tot || o.abs || o.dfl || o.open) return MPDATA_EUNSUPPORTED;
   if (sizeof(T) == 4 && nc == 2)
-    return batched_launch<T, 2>(tab, o, psi_in, psi_out, gc0, gc1, G, R, dt, scale, st);
+    return batched_launch<T, 2>(tab, o, psi_in, psi_out, gc0, gc1, G, R, dt, scale, chained, st);
   if (nc != fused_batched_columns<T>()) return MPDATA_EINVAL;
-  return batched_launch<T, sizeof(T) == 4 ? 4 : 2>(tab, o, psi_in, psi_out, gc0, gc1, G, R, dt, scale, st);
+  return batched_launch<T, sizeof(T) == 4 ? 4 : 2>(tab, o, psi_in, psi_out, gc0, gc1, G, R, dt, scale, chained, st);
 }
 
 template int fused_batched_step<float>(const BatchTable&, const Opts&, const float*, float*, const float*,
-                                       const float*, const float*, const float*, float, float, cudaStream_t, int);
+                                       const float*, const float*, const float*, float, float, bool, cudaStream_t,
+                                       int);
 template int fused_batched_step<double>(const BatchTable&, const Opts&, const double*, double*, const double*,
-                                        const double*, const double*, const double*, double, double, cudaStream_t,
-                                        int);
+                                        const double*, const double*, const double*, double, double, bool,
+                                        cudaStream_t, int);
 
 namespace {
 

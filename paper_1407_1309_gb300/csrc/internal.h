@@ -121,6 +121,10 @@ struct StepArgs {
   const T* r;    // NULL unless an rhs bit
   T dt;
   T gc_scale;    // advector multiplier of this step
+  // the kernel before this step's on the stream is a step of the same call, so only psi_in and
+  // psi_out depend on it: the fused kernels may then be launched as its dependents (the band march
+  // reads the first rows of the advector, G and R while it finishes; launch.cuh)
+  bool chained = false;
 };
 
 // Scratch of the staged path: 16 arrays of n_max elements.

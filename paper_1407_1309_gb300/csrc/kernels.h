@@ -87,13 +87,13 @@ int fused_batched_columns();
 int fused_strip_stride(int nc);
 template <typename T>
 int fused_batched_step(const BatchTable& tab, const Opts& o, const T* psi_in, T* psi_out, const T* gc0,
-                       const T* gc1, const T* G, const T* R, T dt, T scale, cudaStream_t st, int nc);
+                       const T* gc1, const T* G, const T* R, T dt, T scale, bool chained, cudaStream_t st, int nc);
 
 // One step of all fields of a batched handle in one persistent launch
 // (batched.cu); MPDATA_EUNSUPPORTED when not covered.
 template <typename T>
 int batched_step(mpdata_s* h, const T* psi_in, T* psi_out, const T* const* gc, const T* g, const T* r, T dt,
-                 T gc_scale, const Opts& o);
+                 T gc_scale, bool chained, const Opts& o);
 void batched_free(mpdata_s* h);
 
 // Reverse of one step of a single-field handle (adjoint.cu).

@@ -26,6 +26,7 @@
 #include <type_traits>
 
 #include "kernels.h"
+#include "launch.cuh"
 #include "stencil2d.cuh"
 
 namespace mpd {
@@ -61,6 +62,7 @@ struct F2Params {
   T* lo_out;
   T* tape;       // adjoint tape (TAPE only): arrays of tape_n elements
   long long tape_n;
+  bool chained;  // launched as a dependent of the kernel before it (StepArgs::chained)
 };
 
 // One warp marches one tile: the strip `strip` (columns strip*kStride - kLead ...) from
@@ -442,6 +444,8 @@ __global__ void __launch_bounds__(kWarps * 32) k_fused2d(const F2Params<T> p) {
   constexpr int kArr = arrs<COMP>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  if (gridDim.x <= kChainBlocks) grid_release();
+  grid_wait();  // the step before this one, when launched as its dependent
   const long long wid = static_cast<long long>(blockIdx.x) * kWarps + wib;
   if (wid >= static_cast<long long>(p.strips) * p.rowtiles) return;  // whole warp
   const int strip = static_cast<int>(wid % p.strips);
@@ -460,7 +464,8 @@ void launch(const F2Params<T>& p, cudaStream_t st) {
     return cudaFuncSetAttribute(k_fused2d<T, NC, FCT, NUG, IGA, KAHAN, COMP, TAPE, EXT>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) == cudaSuccess;
   });
-  k_fused2d<T, NC, FCT, NUG, IGA, KAHAN, COMP, TAPE, EXT><<<blocks, kWarps * 32, smem, st>>>(p);
+  launch_chained(p.chained, k_fused2d<T, NC, FCT, NUG, IGA, KAHAN, COMP, TAPE, EXT>, dim3(blocks), dim3(kWarps * 32),
+                 smem, st, p);
 }
 
 inline bool al(const void* q, size_t a) { return q == nullptr || (reinterpret_cast<uintptr_t>(q) % a) == 0; }
@@ -506,6 +511,7 @@ F2Params<T> warp_params(const Grid& g, const Opts& o, const StepArgs<T>& a, bool
   p.lo_out = nullptr;
   p.tape = nullptr;
   p.tape_n = 0;
+  p.chained = a.chained;
   return p;
 }
 

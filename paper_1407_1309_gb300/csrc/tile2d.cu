@@ -23,6 +23,7 @@
 #include <cuda_runtime.h>
 
 #include "kernels.h"
+#include "launch.cuh"
 #include "stencil2d.cuh"
 
 namespace mpd {
@@ -46,6 +47,7 @@ struct TileParams {
   int n0, n1, K, reach, H;
   T dt, scale;
   bool open0, open1, tot, abs, dfl, kahan, rhs_a, rhs_b;
+  bool chained;  // launched as a dependent of the kernel before it (StepArgs::chained)
 };
 
 // f(r, c) over rows [r0, r1) x columns [c0, c1), dealt to the threads cell by cell
@@ -121,6 +123,8 @@ __global__ void __launch_bounds__(kThreadsT, 2) k_tile2d(const TileParams<T> p) 
   auto inside = [&](int r, int c) {
     return !(e0 && (x0 + r < 0 || x0 + r >= p.n0)) && !(e1 && (y0 + c < 0 || y0 + c >= p.n1));
   };
+  if (gridDim.x * gridDim.y * gridDim.z <= kChainBlocks) grid_release();
+  grid_wait();
   over(0, kRows + 2 * H, 0, L, [&](int r, int c) {
     if (!inside(r, c)) return;
     int gr = x0 + r, gc = y0 + c;
@@ -305,7 +309,7 @@ int launch_tile(const TileParams<T>& p, int fields, cudaStream_t st) {
   if (smem > static_cast<size_t>(most) || ty > 65535) return MPDATA_EUNSUPPORTED;
   const dim3 grid(static_cast<unsigned>((p.n1 + kCols - 1) / kCols), static_cast<unsigned>(ty),
                   static_cast<unsigned>(fields));
-  k_tile2d<T, FCT, IGA, NUG><<<grid, kThreadsT, smem, st>>>(p);
+  launch_chained(p.chained, k_tile2d<T, FCT, IGA, NUG>, grid, dim3(kThreadsT), smem, st, p);
   return cudaGetLastError() == cudaSuccess ? MPDATA_OK : MPDATA_ECUDA;
 }
 
@@ -340,6 +344,7 @@ int tile2d_step(const Grid& g, const Opts& o, const StepArgs<T>& a, int fields, 
   p.kahan = o.kahan;
   p.rhs_a = o.rhs_a;
   p.rhs_b = o.rhs_b;
+  p.chained = a.chained;
 #define MPD_T(F, I) (o.nug ? launch_tile<T, F, I, true>(p, fields, st) : launch_tile<T, F, I, false>(p, fields, st))
   if (o.fct) return o.iga ? MPD_T(true, true) : MPD_T(true, false);
   return o.iga ? MPD_T(false, true) : MPD_T(false, false);
