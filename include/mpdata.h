@@ -299,7 +299,8 @@ int mpdata_clear_stop(mpdata_t h);
  * MPDATA_TUNE_KERNEL: fused 2D kernel family for single-field 2D steps:
  *   0 = automatic (band march where the warp march cannot fill the GPU: FP32
  *   fields with fewer than ~600 warp tiles of 8 rows, FP64 fields whose warp
- *   tiles would be 16 rows or less; warp march otherwise), 1 = warp march,
+ *   tiles would be 16 rows or less; warp march otherwise, FP32 with lanes of 4 or 2 columns,
+ *   whichever should be faster), 1 = warp march,
  *   2 = band march, 3 = warp march with lanes of 2 columns instead of 4 (FP32; twice
  *   the warps on a small field; for the FP64 fields, whose lanes already own 2, the warp
  *   march).  Batched handles always use the warp march's persistent kernel, with lanes of 2

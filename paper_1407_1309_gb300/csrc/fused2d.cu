@@ -198,6 +198,12 @@ int fused_step(const Grid& g, const Opts& o, const StepArgs<T>& a, T*, cudaStrea
   }
   const F2Params<T> p = warp_params(g, o, a, &band_auto);
   if (o.kernel == 2 || (o.kernel == 0 && band_auto)) return band_step<T>(g, o, a, st);
+  if constexpr (sizeof(T) == 4) {
+    if (o.kernel == 0 && o.tile_rows == 0 && narrow_lanes(p.n0, p.n1, false)) {
+      launch_all<T, 2>(warp_params<T, 2>(g, o, a, &band_auto), o, st);
+      return cudaGetLastError() == cudaSuccess ? MPDATA_OK : MPDATA_ECUDA;
+    }
+  }
   launch_all<T, NC>(p, o, st);
   return cudaGetLastError() == cudaSuccess ? MPDATA_OK : MPDATA_ECUDA;
 }
@@ -207,15 +213,16 @@ int fused_step_comp(const Grid& g, const Opts& o, const StepArgs<float>& a, cons
   if (g.nd != 2 || o.n_iters != 2 || o.tot || o.abs || o.dfl || o.open) return MPDATA_EUNSUPPORTED;
   if (a.psi_out == a.psi_in || lo_out == lo_in) return MPDATA_EUNSUPPORTED;
   bool band_auto = false;
-  if (o.kernel == 3 && o.fct && !o.nug) {  // narrow lanes, the common case
-    F2Params<float> p = warp_params<float, 2>(g, o, a, &band_auto);
+  const bool narrow = o.kernel == 3 || (o.kernel == 0 && o.tile_rows == 0 && narrow_lanes(g.n[1], g.n[2], true));
+  if (narrow && o.fct && !o.nug) {  // lanes of 2 columns, the common case
+    F2Params<float> p = warp_params<float, 2>(g, o, a, &band_auto, true);
     p.lo = lo_in;
     p.lo_out = lo_out;
     p.vec = p.vec && al(lo_in, 8) && al(lo_out, 8);
     launch_comp<true, false, 2>(p, o.iga, st);
     return cudaGetLastError() == cudaSuccess ? MPDATA_OK : MPDATA_ECUDA;
   }
-  F2Params<float> p = warp_params(g, o, a, &band_auto);  // the warp march carries the low parts
+  F2Params<float> p = warp_params(g, o, a, &band_auto, true);  // the warp march carries the low parts
   p.lo = lo_in;
   p.lo_out = lo_out;
   p.vec = p.vec && al(lo_in, 16) && al(lo_out, 16);
@@ -236,6 +243,16 @@ int fused_tape(const Grid& g, const Opts& o, const StepArgs<T>& a, T* tape, cuda
   bool band_auto = false;
   F2Params<T> p = warp_params(g, o, a, &band_auto);
   if (o.kernel == 2 || (o.kernel == 0 && band_auto)) return band_tape<T>(g, o, a, tape, st);
+  if constexpr (sizeof(T) == 4) {  // the lanes that the step itself takes, so that the results are its bits
+    if (o.kernel == 3 || (o.kernel == 0 && o.tile_rows == 0 && narrow_lanes(p.n0, p.n1, false))) {
+      p = warp_params<T, 2>(g, o, a, &band_auto);
+      p.tape = tape;
+      p.tape_n = g.N;
+      if (o.fct) launch<T, 2, true, false, false, false, false, true>(p, st);
+      else launch<T, 2, false, false, false, false, false, true>(p, st);
+      return cudaGetLastError() == cudaSuccess ? MPDATA_OK : MPDATA_ECUDA;
+    }
+  }
   p.tape = tape;
   p.tape_n = g.N;
   if (o.fct) launch<T, NC, true, false, false, false, false, true>(p, st);

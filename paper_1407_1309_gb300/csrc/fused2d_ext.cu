@@ -27,10 +27,8 @@ int fused_step_ext(const Grid& g, const Opts& o, const StepArgs<float>& a, cudaS
   if (g.nd != 2 || o.n_iters != 2 || o.tot || o.iga || o.open || o.kahan) return MPDATA_EUNSUPPORTED;
   if (a.psi_out == a.psi_in) return MPDATA_EUNSUPPORTED;
   bool band_auto = false;
-  // lanes of 2 columns where lanes of 4 leave most of the GPU without a warp (the plain step's rule
-  // for its band march, which these options do not have)
   F2Params<float> p = warp_params(g, o, a, &band_auto);
-  if (o.kernel == 3 || (o.kernel == 0 && band_auto)) {
+  if (o.kernel == 3 || (o.kernel == 0 && o.tile_rows == 0 && narrow_lanes(p.n0, p.n1, false))) {
     p = warp_params<float, 2>(g, o, a, &band_auto);
     if (o.abs && o.dfl) launch_ext<2, kExtAbs | kExtDfl>(p, o, st);
     else if (o.abs) launch_ext<2, kExtAbs>(p, o, st);

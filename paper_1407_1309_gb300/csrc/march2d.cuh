@@ -470,12 +470,53 @@ void launch(const F2Params<T>& p, cudaStream_t st) {
 
 inline bool al(const void* q, size_t a) { return q == nullptr || (reinterpret_cast<uintptr_t>(q) % a) == 0; }
 
+// Tile height of the FP32 warp march and the time it should take.  Every warp of a tile height ty
+// marches ty + 6 rows; with k blocks on the fullest SM one row of all of them takes it c(k)
+// microseconds, more than k times one block's share only while few warps leave the issue slots idle
+// (c measured on fields of 256^2 .. 4096^2: one block takes almost as long as two).  The
+// height is the smallest that keeps the fullest SM at k blocks, for the k of least time.  Against
+// the earlier list of heights (the tallest with 7.5 warps per SM): 4096^2 102 -> 96 us (121 rows
+// instead of 64), 2000 x 500 13.9 -> 10.8 us (with lanes of 2).
+struct MarchRows {
+  int ty;
+  float us;
+};
+template <int NC>
+inline MarchRows march_rows(int n0, int n1, bool comp) {
+  static_assert(NC == 4 || NC == 2, "lanes of 4 or 2 columns");
+  static const float plain4[4] = {0.55f, 0.70f, 1.05f, 1.42f}, plain2[4] = {0.38f, 0.455f, 0.59f, 0.74f};
+  static const float comp4[4] = {0.93f, 0.97f, 1.37f, 1.83f}, comp2[4] = {0.53f, 0.58f, 0.76f, 0.97f};
+  const float* c = NC == 4 ? (comp ? comp4 : plain4) : (comp ? comp2 : plain2);
+  const long long strips = (n1 + stride<NC>() - 1) / stride<NC>();
+  constexpr long long kSms = 152;
+  MarchRows best{n0 > 4 ? n0 : 4, 0.0f};
+  bool any = false;
+  for (long long k = 1; k <= 6; ++k) {
+    const long long tiles = kSms * k * kWarps / strips;
+    if (tiles < 1) continue;
+    long long ty = (n0 + tiles - 1) / tiles;
+    if (ty < 4) ty = 4;
+    const long long blocks = (strips * ((n0 + ty - 1) / ty) + kWarps - 1) / kWarps;
+    const long long full = (blocks + kSms - 1) / kSms;
+    const float us = static_cast<float>(ty + 6) * (full <= 4 ? c[full - 1] : 0.25f * c[3] * static_cast<float>(full));
+    if (!any || us < best.us) best = {static_cast<int>(ty), us};
+    any = true;
+  }
+  return best;
+}
+
+// Whether lanes of 2 columns suit an FP32 field better than lanes of 4: where the narrower strips
+// leave fewer padded columns or, on a field too small to fill the GPU, their twice as many warps
+// hide more latency (compensated 512^2 12.1 -> 8.1 us, plain 2000 x 500 13.9 -> 10.8).
+inline bool narrow_lanes(int n0, int n1, bool comp) {
+  return march_rows<2>(n0, n1, comp).us < 0.98f * march_rows<4>(n0, n1, comp).us;
+}
+
 // Warp-march parameters of one step of one field; *band is set when the automatic choice is
-// the band march.  NC columns per lane: FP32 lanes own 4 (16-byte copies) or, with
-// MPDATA_TUNE_KERNEL = 3, 2 (twice the strips, so twice the warps on a small field), FP64
-// lanes 2 (register budget).
+// the band march.  NC columns per lane: FP32 lanes own 4 (16-byte copies) or 2 (narrow_lanes, or
+// MPDATA_TUNE_KERNEL = 3), FP64 lanes 2 (register budget).
 template <typename T, int NC = (sizeof(T) == 4 ? 4 : 2)>
-F2Params<T> warp_params(const Grid& g, const Opts& o, const StepArgs<T>& a, bool* band) {
+F2Params<T> warp_params(const Grid& g, const Opts& o, const StepArgs<T>& a, bool* band, bool comp = false) {
   F2Params<T> p;
   p.psi = a.psi_in;
   p.out = a.psi_out;
@@ -486,12 +527,14 @@ F2Params<T> warp_params(const Grid& g, const Opts& o, const StepArgs<T>& a, bool
   p.n0 = g.n[1];
   p.n1 = g.n[2];
   p.strips = (p.n1 + stride<NC>() - 1) / stride<NC>();
-  // the tallest tile that still gives ~7.5 warps per SM (152 SMs), at least 8 rows
-  // (measured on the rotation workload: 8 rows at 1024^2, 32 at 2048^2, 48-64 at 4096^2)
   auto warps = [&](int ty) { return static_cast<long long>(p.strips) * ((p.n0 + ty - 1) / ty); };
   int auto_ty = 8;
-  for (int ty : {64, 48, 32, 24, 16, 12}) {
-    if (warps(ty) >= 1140) { auto_ty = ty; break; }
+  if constexpr (sizeof(T) == 4) {
+    auto_ty = march_rows<NC>(p.n0, p.n1, comp).ty;
+  } else {  // FP64: the tallest tile that still gives ~7.5 warps per SM (152 SMs), at least 8 rows
+    for (int ty : {64, 48, 32, 24, 16, 12}) {
+      if (warps(ty) >= 1140) { auto_ty = ty; break; }
+    }
   }
   // Where the warp march cannot fill the GPU even with 8-row tiles (FP32: fewer than ~4
   // warps per SM), or in FP64 (arithmetic-bound: every recomputed halo row costs FP64
