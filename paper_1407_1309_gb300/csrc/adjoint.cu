@@ -699,7 +699,7 @@ int adjoint_nd(mpdata_s* h, const Grid& g, const Opts& o, const T* psi_n, const 
     if constexpr (ND == 2) {
       // 2D: one launch of the fused step writes the tape and the step's result
       if (!o.staged && psi_next) {
-        const StepArgs<T> a{psi_n, psi_next, {gc[0], gc[1], nullptr}, nullptr, nullptr, T(0), T(1)};
+        const StepArgs<T> a{psi_n, psi_next, {gc[0], gc[1], nullptr}, nullptr, nullptr, T(0), T(1), true};
         const int rc = fused_tape<T>(g, o, a, tape, st);
         if (rc != MPDATA_EUNSUPPORTED) return rc;
       }
@@ -775,7 +775,7 @@ int adjoint_nd(mpdata_s* h, const Grid& g, const Opts& o, const T* psi_n, const 
     if constexpr (ND == 2) {
       if (!o.staged) {
         T* const unused = tape_base + tape_arrays(K, D, o.fct) * static_cast<size_t>(N);
-        const StepArgs<T> a{psi_n, unused, {gc[0], gc[1], nullptr}, nullptr, nullptr, T(0), T(1)};
+        const StepArgs<T> a{psi_n, unused, {gc[0], gc[1], nullptr}, nullptr, nullptr, T(0), T(1), true};
         rc = fused_tape<T>(g, o, a, tape_base, st);
       }
     }

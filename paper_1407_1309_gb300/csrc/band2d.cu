@@ -50,6 +50,7 @@ struct BandParams {
   long long tape_n;
   int tape_vec;  // tape rows may be written as 16-byte vectors
   bool chained;  // launched as a dependent of the kernel before it (StepArgs::chained)
+  bool early;    // the advector, G and R may be read before that kernel is complete (StepArgs::early)
 };
 
 // NC values of one lane from / to a shared-memory row (16-byte vectors where they fit)
@@ -178,6 +179,7 @@ __global__ void __launch_bounds__(W * 32, 2) k_band2d(const BandParams<T> p) {
   // the first chunks: what no earlier step of the call writes, then, once the step before this one
   // is complete, psi (the copies of the first part join the first chunk's group)
   if (gridDim.x <= kChainBlocks) grid_release();
+  if (!p.early) grid_wait();
 #pragma unroll
   for (int j = 0; j < kDepth; ++j) load_row(j * W + w, kRest);
   g_row = wrapi(Rs + w, p.n0);
@@ -510,6 +512,7 @@ int band_step(const Grid& g, const Opts& o, const StepArgs<T>& a, cudaStream_t s
   p.tape_n = 0;
   p.tape_vec = 0;
   p.chained = a.chained;
+  p.early = a.early;
   if (o.fct) {
     if (o.nug) band_mode<T, NC, true, true>(p, o.tile_rows, o.iga, o.kahan, st);
     else band_mode<T, NC, true, false>(p, o.tile_rows, o.iga, o.kahan, st);
@@ -547,6 +550,7 @@ int band_tape(const Grid& g, const Opts& o, const StepArgs<T>& a, T* tape, cudaS
   p.tape_n = g.N;
   p.tape_vec = p.vec && aligned_to(tape, 16);
   p.chained = a.chained;
+  p.early = a.early;
   if (o.fct) launch_band<T, NC, true, false, false, false, true>(p, o.tile_rows, st);
   else launch_band<T, NC, false, false, false, false, true>(p, o.tile_rows, st);
   return cudaGetLastError() == cudaSuccess ? MPDATA_OK : MPDATA_ECUDA;

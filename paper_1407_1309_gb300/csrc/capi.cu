@@ -88,11 +88,11 @@ int run_trapez(mpdata_s* h, const T* psi_in, T* psi_out, const void* const* gcv,
   T* S = static_cast<T*>(h->trapez_buf);
   for (int s = 0; s < n_steps; ++s) {
     if (h->stop.load(std::memory_order_relaxed)) return MPDATA_ESTOPPED;
-    if (mpd::trapez_pre<T>(m, n, static_cast<T>(dt), s == 0 ? psi_in : psi_out, b, S, h->stream) != cudaSuccess)
+    if (mpd::trapez_pre<T>(m, n, static_cast<T>(dt), s == 0 ? psi_in : psi_out, b, S, s > 0, h->stream) != cudaSuccess)
       return MPDATA_ECUDA;
     const int rc = run_advance<T>(h, S, psi_out, gcv, g, nullptr, dt, 1, gc_scale ? gc_scale + s : nullptr, true);
     if (rc != MPDATA_OK) return rc;
-    if (mpd::trapez_post<T>(m, n, static_cast<T>(dt), b, psi_out, h->stream) != cudaSuccess) return MPDATA_ECUDA;
+    if (mpd::trapez_post<T>(m, n, static_cast<T>(dt), b, psi_out, true, h->stream) != cudaSuccess) return MPDATA_ECUDA;
   }
   return MPDATA_OK;
 }
@@ -149,8 +149,9 @@ int run_advance(mpdata_s* h, const T* psi_in, T* psi_out, const void* const* gcv
       return MPDATA_ECUDA;
     cur = P;
   }
-  // whether the last kernel on the stream is a fused step of this call (StepArgs::chained)
-  bool chained = false;
+  // whether the last kernel on the stream belongs to this call (StepArgs::chained; none of them writes
+  // the advector, G or R)
+  bool chained = inner;
   for (int s = 0; s < n_steps; ++s) {
     if (h->stop.load(std::memory_order_relaxed)) return MPDATA_ESTOPPED;
     const T scale = gc_scale ? static_cast<T>(gc_scale[s]) : T(1);
@@ -176,9 +177,10 @@ int run_advance(mpdata_s* h, const T* psi_in, T* psi_out, const void* const* gcv
       a.dt = static_cast<T>(dt);
       a.gc_scale = scale;
       a.chained = chained;
+      a.early = chained;
       int rc = o.staged ? MPDATA_EUNSUPPORTED : mpd::fused_step<T>(gr, o, a, nullptr, h->stream);
       if (rc == MPDATA_EUNSUPPORTED && !o.staged) rc = mpd::tile2d_step<T>(gr, o, a, 1, 0, h->stream);
-      chained = rc == MPDATA_OK;
+      chained = true;
       if (rc == MPDATA_EUNSUPPORTED) rc = cuda_status(mpd::staged_step<T>(gr, o, a, ss, h->stream));
       if (rc != MPDATA_OK) return rc;
     }
@@ -284,10 +286,10 @@ int run_sw(mpdata_s* h, T* state, double dt, double dx, double eps, int n_steps)
     if (h->stop.load(std::memory_order_relaxed)) return MPDATA_ESTOPPED;
     T* dst = ((n_steps - 1 - s) % 2 == 0) ? X : P;
     if (mpd::vip_advector<T>(gr, cur, uprev, ext, adv, h->sw_first, static_cast<T>(eps), static_cast<T>(dt / dx),
-                             h->stream) != cudaSuccess)
+                             s > 0, h->stream) != cudaSuccess)
       return MPDATA_ECUDA;
     h->sw_first = false;
-    if (mpd::sw_force<T>(gr, cur, static_cast<T>(0.5 * dt), static_cast<T>(dx), h->stream) != cudaSuccess)
+    if (mpd::sw_force<T>(gr, cur, static_cast<T>(0.5 * dt), static_cast<T>(dx), true, h->stream) != cudaSuccess)
       return MPDATA_ECUDA;
     // every field by the fused march where that covers the options, else all fields in one launch
     // of the tile kernel (2D), else field by field on the staged kernels
@@ -300,6 +302,7 @@ int run_sw(mpdata_s* h, T* state, double dt, double dx, double eps, int n_steps)
       a.r = nullptr;
       a.dt = static_cast<T>(dt);
       a.gc_scale = T(1);
+      a.chained = true;  // the advector was written two kernels before: not read early
       int rc = o.staged ? MPDATA_EUNSUPPORTED : mpd::fused_step<T>(gr, o, a, nullptr, h->stream);
       if (rc == MPDATA_EUNSUPPORTED && !o.staged && f == 0) {
         rc = mpd::tile2d_step<T>(gr, o, a, nd + 1, n, h->stream);
@@ -308,7 +311,7 @@ int run_sw(mpdata_s* h, T* state, double dt, double dx, double eps, int n_steps)
       if (rc == MPDATA_EUNSUPPORTED) rc = cuda_status(mpd::staged_step<T>(gr, o, a, ss, h->stream));
       if (rc != MPDATA_OK) return rc;
     }
-    if (mpd::sw_force<T>(gr, dst, static_cast<T>(0.5 * dt), static_cast<T>(dx), h->stream) != cudaSuccess)
+    if (mpd::sw_force<T>(gr, dst, static_cast<T>(0.5 * dt), static_cast<T>(dx), true, h->stream) != cudaSuccess)
       return MPDATA_ECUDA;
     cur = dst;
   }
@@ -448,6 +451,7 @@ int mpdata_advance_compensated(mpdata_t h, const void* psi_in, const void* lo_in
     a.dt = static_cast<float>(dt);
     a.gc_scale = gc_scale ? static_cast<float>(gc_scale[s]) : 1.0f;
     a.chained = s > 0;
+    a.early = s > 0;
     rc = mpd::fused_step_comp(h->grids[0], o, a, curl, dstl, h->stream);
     if (rc != MPDATA_OK) return rc;
     cur = dst;

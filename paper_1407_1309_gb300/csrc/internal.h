@@ -121,10 +121,12 @@ struct StepArgs {
   const T* r;    // NULL unless an rhs bit
   T dt;
   T gc_scale;    // advector multiplier of this step
-  // the kernel before this step's on the stream is a step of the same call, so only psi_in and
-  // psi_out depend on it: the fused kernels may then be launched as its dependents (the band march
-  // reads the first rows of the advector, G and R while it finishes; launch.cuh)
+  // the kernel before this step's on the stream belongs to the same call: the step's first kernel is
+  // launched as its dependent (launch.cuh)
   bool chained = false;
+  // and no kernel that such a dependent may start before writes the advector, G or R, so that they
+  // may be read while the kernel before it finishes
+  bool early = false;
 };
 
 // Scratch of the staged path: 16 arrays of n_max elements.
@@ -199,25 +201,25 @@ cudaError_t staged_forward_tape(const Grid& g, const Opts& o, const T* const* gc
                                 const Tape<T>& tp, T* const* psi_out_levels, T* psi_next, cudaStream_t st);
 
 template <typename T>
-cudaError_t trapez_pre(const TrapezMat& m, long long n, T dt, const T* psi, const T* b, T* out, cudaStream_t st);
+cudaError_t trapez_pre(const TrapezMat& m, long long n, T dt, const T* psi, const T* b, T* out, bool chained, cudaStream_t st);
 template <typename T>
-cudaError_t trapez_post(const TrapezMat& m, long long n, T dt, const T* b, T* psi, cudaStream_t st);
+cudaError_t trapez_post(const TrapezMat& m, long long n, T dt, const T* b, T* psi, bool chained, cudaStream_t st);
 
 // Vectorised FP32 pseudo-advector z-march for 3D fields (march3.cu): launched, and true
-// returned, when the x extent is a multiple of 4 and at least 128, no edge is open and every
-// array is 16-byte aligned; false (nothing launched) otherwise.
+// returned, when the x extent is at least 48 and no edge is open; false (nothing launched)
+// otherwise.  chained: as a dependent of the kernel before it (launch.cuh).
 bool antidiff3_vec(const Grid& g, const float* psi, const float* const* v, float vscale, const float* G, bool iga,
-                   bool tot, bool abs_psi, float* const* out, cudaStream_t st);
+                   bool tot, bool abs_psi, float* const* out, bool chained, cudaStream_t st);
 
 // Vectorised FP32 pass-1-and-bounds z-march (march3.cu), same conditions.
 bool p1b3_vec(const Grid& g, const float* psi, const float* const* v, float vscale, const float* G, bool kahan,
-              float* p1, float* mx, float* mn, cudaStream_t st);
+              float* p1, float* mx, float* mn, bool chained, cudaStream_t st);
 
 // Vectorised FP32 FCT corrective pass (march3.cu): factors, limiter and donor pass as one z-march,
 // same conditions, and neither the Kahan summation nor a source term (post); lim[0] null when the
 // limited advector is not wanted.
 bool corr3_vec(const Grid& g, const float* psi, const float* const* vu, const float* G, bool iga, bool kahan,
-               const float* mx, const float* mn, bool post, float* const* lim, float* out, cudaStream_t st);
+               const float* mx, const float* mn, bool post, float* const* lim, float* out, bool chained, cudaStream_t st);
 
 // Prognosed velocity and shallow-water sources (vip.cu).  state: h then the momenta q_d, n cells
 // each.  vip_advector: the advector of the step (adv, nd arrays) from the velocities q/h (h > eps)
@@ -226,9 +228,9 @@ bool corr3_vec(const Grid& g, const float* psi, const float* const* vu, const fl
 // R_d = -h dh/dx_d by centred differences.
 template <typename T>
 cudaError_t vip_advector(const Grid& g, const T* state, T* uprev, T* ext, T* adv, bool first, T eps, T courant,
-                         cudaStream_t st);
+                         bool chained, cudaStream_t st);
 template <typename T>
-cudaError_t sw_force(const Grid& g, T* state, T half_dt, T dx, cudaStream_t st);
+cudaError_t sw_force(const Grid& g, T* state, T half_dt, T dx, bool chained, cudaStream_t st);
 
 // FP64 reductions (reduce.cu).  partial: device scratch of at least
 // kRedBlocks * n_fields doubles per output.

@@ -30,28 +30,28 @@ bool chunks(const Grid& g, const float* const* v, const float* const* w) {
 }  // namespace
 
 bool antidiff3_vec(const Grid& g, const float* psi, const float* const* v, float vscale, const float* G, bool iga,
-                   bool tot, bool abs_psi, float* const* out, cudaStream_t st) {
+                   bool tot, bool abs_psi, float* const* out, bool chained, cudaStream_t st) {
   if (!use_vec(g)) return false;
-  if (chunks(g, v, out) && al16(psi) && al16(G)) antidiff3_nc<4, true>(g, psi, v, vscale, G, iga, tot, abs_psi, out, st);
-  else antidiff3_cells(g, psi, v, vscale, G, iga, tot, abs_psi, out, st);
+  if (chunks(g, v, out) && al16(psi) && al16(G)) antidiff3_nc<4, true>(g, psi, v, vscale, G, iga, tot, abs_psi, out, chained, st);
+  else antidiff3_cells(g, psi, v, vscale, G, iga, tot, abs_psi, out, chained, st);
   return true;
 }
 
 bool p1b3_vec(const Grid& g, const float* psi, const float* const* v, float vscale, const float* G, bool kahan,
-              float* p1, float* mx, float* mn, cudaStream_t st) {
+              float* p1, float* mx, float* mn, bool chained, cudaStream_t st) {
   if (!use_vec(g)) return false;
   const float* const o[3] = {p1, mx, mn};
-  if (chunks(g, v, o) && al16(psi) && al16(G)) p1b3_nc<4, true>(g, psi, v, vscale, G, kahan, p1, mx, mn, st);
-  else p1b3_cells(g, psi, v, vscale, G, kahan, p1, mx, mn, st);
+  if (chunks(g, v, o) && al16(psi) && al16(G)) p1b3_nc<4, true>(g, psi, v, vscale, G, kahan, p1, mx, mn, chained, st);
+  else p1b3_cells(g, psi, v, vscale, G, kahan, p1, mx, mn, chained, st);
   return true;
 }
 
 bool corr3_vec(const Grid& g, const float* psi, const float* const* vu, const float* G, bool iga, bool kahan,
-               const float* mx, const float* mn, bool post, float* const* lim, float* out, cudaStream_t st) {
+               const float* mx, const float* mn, bool post, float* const* lim, float* out, bool chained, cudaStream_t st) {
   if (!use_vec(g) || kahan || post) return false;
   if (chunks(g, vu, lim) && al16(psi) && al16(G) && al16(mx) && al16(mn) && al16(out))
-    corr3_nc<4, true>(g, psi, vu, G, iga, mx, mn, lim, out, st);
-  else corr3_cells(g, psi, vu, G, iga, mx, mn, lim, out, st);
+    corr3_nc<4, true>(g, psi, vu, G, iga, mx, mn, lim, out, chained, st);
+  else corr3_cells(g, psi, vu, G, iga, mx, mn, lim, out, chained, st);
   return true;
 }
 

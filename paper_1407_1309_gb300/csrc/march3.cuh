@@ -21,6 +21,7 @@
 #include <type_traits>
 
 #include "internal.h"
+#include "launch.cuh"
 #include "stencil2d.cuh"
 
 namespace mpd {
@@ -232,6 +233,7 @@ __global__ void __launch_bounds__(kThreads, MINB) k_antidiff3v(Grid g, int zc_an
   // ring slots at step z: psi planes z-1 .. z+2 in cp .. cp+3; z component planes z-1, z in
   // cz, cz+1; y, x components and G planes z, z+1 in cq, cq+1
   int cp = 0, cz = 0, cq = 0;
+  grid_wait();
   {  // prologue
     for (int j = 0; j < 4; ++j) pp.copy(sP + j * nP, psi + zoff(zb - 1 + j), tid);
     pv.copy(sZ, Vin.p[0] + zoff(zb - 1), tid);
@@ -463,6 +465,7 @@ __global__ void __launch_bounds__(kCThreads, 2) k_p1b3v(Grid g, int zc_any, cons
   auto Yp = [&](int j) { return sY + rj(kq, j, kBVqRing) * nY; };
   auto Zp = [&](int j) { return sZ + rj(kz, j, kBVzRing) * nZ; };
   auto Qp = [&](int j) { return s1 + rj(k1, j, kB1Ring) * n1; };
+  grid_wait();
   {  // prologue (step zb-1): psi^n planes zb-2 .. zb, z component zb-2, zb-1, x and y components zb-1
     for (int j = -1; j <= 1; ++j) pn.copy(Np(j), psi + zoff(zb - 1 + j), tid);
     pz.copy(Zp(-1), V.p[0] + zoff(zb - 2), tid);
@@ -719,6 +722,7 @@ __global__ void __launch_bounds__(kCThreads, 2) k_corr3v(Grid g, int zc_any, con
   float vz_n[NC], vz_c[NC], vz_m[NC], vz_mm[NC], mx_n[NC], mn_n[NC], g_n[NC], g_c[NC], g_m[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) { vz_m[c] = 0.0f; g_c[c] = 1.0f; g_n[c] = 1.0f; }
+  grid_wait();
   {  // prologue (step zb-1): psi planes zb-2 .. zb, components of plane zb-1
     pp.copy(sP + 1 * nP, psi + zoff(zb - 2), tid);
     pp.copy(sP + 2 * nP, psi + zoff(zb - 1), tid);
@@ -944,7 +948,7 @@ inline void want_smem(PerDevice<bool>& attr, K kern, size_t bytes) {
 
 template <int NC, int MINB, bool VEC, bool ABS, bool IGA, bool TOT, bool NUG>
 void launch_v(const Grid& g, const float* psi, const float* const* v, float vscale, const float* G, float* const* out,
-              cudaStream_t st) {
+              bool chained, cudaStream_t st) {
   const int zc = z_chunk<NC>(g);
   V3 vin{{v[0], v[1], v[2]}};
   O3 vo{{out[0], out[1], out[2]}};
@@ -952,26 +956,26 @@ void launch_v(const Grid& g, const float* psi, const float* const* v, float vsca
     auto kern = k_antidiff3v<NC, MINB, VEC, decltype(c)::value, ABS, IGA, TOT, NUG>;
     static PerDevice<bool> attr;
     want_smem(attr, kern, antidiff3v_smem<NC>());
-    kern<<<march_grid<NC>(g, zc), dim3(32, kRows), antidiff3v_smem<NC>(), st>>>(g, zc, psi, vin, vscale, G, vo);
+    launch_chained(chained, kern, march_grid<NC>(g, zc), dim3(32, kRows), antidiff3v_smem<NC>(), st, g, zc, psi, vin, vscale, G, vo);
   });
 }
 
 template <int NC, bool VEC, bool KAHAN, bool NUG>
 void launch_b(const Grid& g, const float* psi, const float* const* v, float vscale, const float* G, float* p1,
-              float* mx, float* mn, cudaStream_t st) {
+              float* mx, float* mn, bool chained, cudaStream_t st) {
   const int zc = z_chunk<NC>(g);
   V3 vv{{v[0], v[1], v[2]}};
   with_chunk<VEC>(zc, [&](auto c) {
     auto kern = k_p1b3v<NC, VEC, decltype(c)::value, KAHAN, NUG>;
     static PerDevice<bool> attr;
     want_smem(attr, kern, p1b3v_smem<NC>());
-    kern<<<march_grid<NC>(g, zc), dim3(32, kCWarps), p1b3v_smem<NC>(), st>>>(g, zc, psi, vv, vscale, G, p1, mx, mn);
+    launch_chained(chained, kern, march_grid<NC>(g, zc), dim3(32, kCWarps), p1b3v_smem<NC>(), st, g, zc, psi, vv, vscale, G, p1, mx, mn);
   });
 }
 
 template <int NC, bool VEC, bool NUG, bool UNIT, bool LIM>
 void launch_k(const Grid& g, const float* psi, const float* const* vu, const float* G, const float* mx,
-              const float* mn, float* const* lim, float* out, cudaStream_t st) {
+              const float* mn, float* const* lim, float* out, bool chained, cudaStream_t st) {
   const int zc = z_chunk<NC>(g);
   V3 vv{{vu[0], vu[1], vu[2]}};
   O3 lo{{lim[0], lim[1], lim[2]}};
@@ -979,14 +983,14 @@ void launch_k(const Grid& g, const float* psi, const float* const* vu, const flo
     auto kern = k_corr3v<NC, VEC, decltype(c)::value, NUG, UNIT, LIM>;
     static PerDevice<bool> attr;
     want_smem(attr, kern, corr3v_smem<NC>());
-    kern<<<march_grid<NC>(g, zc), dim3(32, kCWarps), corr3v_smem<NC>(), st>>>(g, zc, psi, vv, G, mx, mn, lo, out);
+    launch_chained(chained, kern, march_grid<NC>(g, zc), dim3(32, kCWarps), corr3v_smem<NC>(), st, g, zc, psi, vv, G, mx, mn, lo, out);
   });
 }
 
 template <int NC, bool VEC>
 void antidiff3_nc(const Grid& g, const float* psi, const float* const* v, float vscale, const float* G, bool iga,
-                  bool tot, bool abs_psi, float* const* out, cudaStream_t st) {
-#define MPD_V(A, I, T, N) launch_v<NC, 2, VEC, A, I, T, N>(g, psi, v, vscale, G, out, st)
+                  bool tot, bool abs_psi, float* const* out, bool chained, cudaStream_t st) {
+#define MPD_V(A, I, T, N) launch_v<NC, 2, VEC, A, I, T, N>(g, psi, v, vscale, G, out, chained, st)
 #define MPD_VN(A, I, T) \
   do { if (G) MPD_V(A, I, T, true); else MPD_V(A, I, T, false); } while (0)
 #define MPD_VT(A, I) \
@@ -1001,21 +1005,21 @@ void antidiff3_nc(const Grid& g, const float* psi, const float* const* v, float 
 
 template <int NC, bool VEC>
 void p1b3_nc(const Grid& g, const float* psi, const float* const* v, float vscale, const float* G, bool kahan,
-             float* p1, float* mx, float* mn, cudaStream_t st) {
+             float* p1, float* mx, float* mn, bool chained, cudaStream_t st) {
   if (kahan) {
-    if (G) launch_b<NC, VEC, true, true>(g, psi, v, vscale, G, p1, mx, mn, st);
-    else launch_b<NC, VEC, true, false>(g, psi, v, vscale, G, p1, mx, mn, st);
+    if (G) launch_b<NC, VEC, true, true>(g, psi, v, vscale, G, p1, mx, mn, chained, st);
+    else launch_b<NC, VEC, true, false>(g, psi, v, vscale, G, p1, mx, mn, chained, st);
   } else {
-    if (G) launch_b<NC, VEC, false, true>(g, psi, v, vscale, G, p1, mx, mn, st);
-    else launch_b<NC, VEC, false, false>(g, psi, v, vscale, G, p1, mx, mn, st);
+    if (G) launch_b<NC, VEC, false, true>(g, psi, v, vscale, G, p1, mx, mn, chained, st);
+    else launch_b<NC, VEC, false, false>(g, psi, v, vscale, G, p1, mx, mn, chained, st);
   }
 }
 
 template <int NC, bool VEC>
 void corr3_nc(const Grid& g, const float* psi, const float* const* vu, const float* G, bool iga, const float* mx,
-              const float* mn, float* const* lim, float* out, cudaStream_t st) {
+              const float* mn, float* const* lim, float* out, bool chained, cudaStream_t st) {
   const bool lm = lim[0] != nullptr;
-#define MPD_K(N, U, L) launch_k<NC, VEC, N, U, L>(g, psi, vu, G, mx, mn, lim, out, st)
+#define MPD_K(N, U, L) launch_k<NC, VEC, N, U, L>(g, psi, vu, G, mx, mn, lim, out, chained, st)
 #define MPD_KL(N, U) \
   do { if (lm) MPD_K(N, U, true); else MPD_K(N, U, false); } while (0)
   if (G) { if (iga) MPD_KL(true, true); else MPD_KL(true, false); }
@@ -1028,10 +1032,10 @@ void corr3_nc(const Grid& g, const float* psi, const float* const* vu, const flo
 
 // The forms for fields whose rows cannot be moved in 16-byte chunks (march3u.cu).
 void antidiff3_cells(const Grid& g, const float* psi, const float* const* v, float vscale, const float* G, bool iga,
-                     bool tot, bool abs_psi, float* const* out, cudaStream_t st);
+                     bool tot, bool abs_psi, float* const* out, bool chained, cudaStream_t st);
 void p1b3_cells(const Grid& g, const float* psi, const float* const* v, float vscale, const float* G, bool kahan,
-                float* p1, float* mx, float* mn, cudaStream_t st);
+                float* p1, float* mx, float* mn, bool chained, cudaStream_t st);
 void corr3_cells(const Grid& g, const float* psi, const float* const* vu, const float* G, bool iga, const float* mx,
-                 const float* mn, float* const* lim, float* out, cudaStream_t st);
+                 const float* mn, float* const* lim, float* out, bool chained, cudaStream_t st);
 
 }  // namespace mpd

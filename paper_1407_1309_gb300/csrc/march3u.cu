@@ -22,21 +22,21 @@ bool narrow(const Grid& g) {
 }  // namespace
 
 void antidiff3_cells(const Grid& g, const float* psi, const float* const* v, float vscale, const float* G, bool iga,
-                     bool tot, bool abs_psi, float* const* out, cudaStream_t st) {
-  if (narrow(g)) antidiff3_nc<2, false>(g, psi, v, vscale, G, iga, tot, abs_psi, out, st);
-  else antidiff3_nc<4, false>(g, psi, v, vscale, G, iga, tot, abs_psi, out, st);
+                     bool tot, bool abs_psi, float* const* out, bool chained, cudaStream_t st) {
+  if (narrow(g)) antidiff3_nc<2, false>(g, psi, v, vscale, G, iga, tot, abs_psi, out, chained, st);
+  else antidiff3_nc<4, false>(g, psi, v, vscale, G, iga, tot, abs_psi, out, chained, st);
 }
 
 void p1b3_cells(const Grid& g, const float* psi, const float* const* v, float vscale, const float* G, bool kahan,
-                float* p1, float* mx, float* mn, cudaStream_t st) {
-  if (narrow(g)) p1b3_nc<2, false>(g, psi, v, vscale, G, kahan, p1, mx, mn, st);
-  else p1b3_nc<4, false>(g, psi, v, vscale, G, kahan, p1, mx, mn, st);
+                float* p1, float* mx, float* mn, bool chained, cudaStream_t st) {
+  if (narrow(g)) p1b3_nc<2, false>(g, psi, v, vscale, G, kahan, p1, mx, mn, chained, st);
+  else p1b3_nc<4, false>(g, psi, v, vscale, G, kahan, p1, mx, mn, chained, st);
 }
 
 void corr3_cells(const Grid& g, const float* psi, const float* const* vu, const float* G, bool iga, const float* mx,
-                 const float* mn, float* const* lim, float* out, cudaStream_t st) {
-  if (narrow(g)) corr3_nc<2, false>(g, psi, vu, G, iga, mx, mn, lim, out, st);
-  else corr3_nc<4, false>(g, psi, vu, G, iga, mx, mn, lim, out, st);
+                 const float* mn, float* const* lim, float* out, bool chained, cudaStream_t st) {
+  if (narrow(g)) corr3_nc<2, false>(g, psi, vu, G, iga, mx, mn, lim, out, chained, st);
+  else corr3_nc<4, false>(g, psi, vu, G, iga, mx, mn, lim, out, chained, st);
 }
 
 }  // namespace mpd

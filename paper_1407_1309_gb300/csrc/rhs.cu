@@ -10,6 +10,7 @@
 #include <cmath>
 
 #include "internal.h"
+#include "launch.cuh"
 
 namespace mpd {
 namespace {
@@ -17,6 +18,7 @@ namespace {
 template <typename T>
 __global__ void k_trapez_pre(const TrapezMat m, long long n, T half_dt, const T* __restrict__ psi,
                              const T* __restrict__ b, T* __restrict__ out) {
+  dev::grid_wait();
   for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
        i += static_cast<long long>(gridDim.x) * blockDim.x) {
     T x[kTrapezMax];
@@ -38,6 +40,7 @@ __global__ void k_trapez_pre(const TrapezMat m, long long n, T half_dt, const T*
 template <typename T>
 __global__ void k_trapez_post(const TrapezMat m, long long n, T half_dt, const T* __restrict__ b,
                               T* __restrict__ psi) {
+  dev::grid_wait();
   for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
        i += static_cast<long long>(gridDim.x) * blockDim.x) {
     T y[kTrapezMax];
@@ -100,22 +103,22 @@ bool trapez_matrix(TrapezMat& m, const double* A, int E, double dt) {
 }
 
 template <typename T>
-cudaError_t trapez_pre(const TrapezMat& m, long long n, T dt, const T* psi, const T* b, T* out, cudaStream_t st) {
-  k_trapez_pre<T><<<blocks_for(n), 256, 0, st>>>(m, n, T(0.5) * dt, psi, b, out);
+cudaError_t trapez_pre(const TrapezMat& m, long long n, T dt, const T* psi, const T* b, T* out, bool chained, cudaStream_t st) {
+  launch_chained(chained, k_trapez_pre<T>, dim3(blocks_for(n)), dim3(256), 0, st, m, n, T(0.5) * dt, psi, b, out);
   return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t trapez_post(const TrapezMat& m, long long n, T dt, const T* b, T* psi, cudaStream_t st) {
-  k_trapez_post<T><<<blocks_for(n), 256, 0, st>>>(m, n, T(0.5) * dt, b, psi);
+cudaError_t trapez_post(const TrapezMat& m, long long n, T dt, const T* b, T* psi, bool chained, cudaStream_t st) {
+  launch_chained(chained, k_trapez_post<T>, dim3(blocks_for(n)), dim3(256), 0, st, m, n, T(0.5) * dt, b, psi);
   return cudaGetLastError();
 }
 
 template cudaError_t trapez_pre<float>(const TrapezMat&, long long, float, const float*, const float*, float*,
-                                       cudaStream_t);
+                                       bool, cudaStream_t);
 template cudaError_t trapez_pre<double>(const TrapezMat&, long long, double, const double*, const double*, double*,
-                                        cudaStream_t);
-template cudaError_t trapez_post<float>(const TrapezMat&, long long, float, const float*, float*, cudaStream_t);
-template cudaError_t trapez_post<double>(const TrapezMat&, long long, double, const double*, double*, cudaStream_t);
+                                        bool, cudaStream_t);
+template cudaError_t trapez_post<float>(const TrapezMat&, long long, float, const float*, float*, bool, cudaStream_t);
+template cudaError_t trapez_post<double>(const TrapezMat&, long long, double, const double*, double*, bool, cudaStream_t);
 
 }  // namespace mpd

@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include "internal.h"
+#include "launch.cuh"
 #include "stencil2d.cuh"
 
 namespace mpd {
@@ -154,6 +155,7 @@ __device__ __forceinline__ T flux(T L, T R, T V, bool unit) {
 template <typename T>
 __global__ void k_pre(long long N, const T* __restrict__ psi, const T* __restrict__ r, T dt,
                       T* __restrict__ out) {
+  dev::grid_wait();
   const long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
   if (i < N) out[i] = psi[i] + dt * r[i];
 }
@@ -164,6 +166,7 @@ template <typename T, int ND>
 __global__ void k_donor(Grid g, const T* __restrict__ psi, In3<T> V, T vscale, bool unit,
                         const T* __restrict__ G, bool kahan, const T* __restrict__ R, T dt,
                         bool post, T* __restrict__ out) {
+  dev::grid_wait();
   FOR_CELLS(g) {
   const Nbr<ND> nb(g, Coord{{c0_, c1_, c2_}});
   const long long i = nb.i;
@@ -202,6 +205,7 @@ __global__ void k_donor(Grid g, const T* __restrict__ psi, In3<T> V, T vscale, b
 template <typename T, int ND>
 __global__ void k_bounds(Grid g, const T* __restrict__ p0, const T* __restrict__ p1,
                          T* __restrict__ mx, T* __restrict__ mn) {
+  dev::grid_wait();
   FOR_CELLS(g) {
   const Nbr<ND> nb(g, Coord{{c0_, c1_, c2_}});
   const long long i = nb.i;
@@ -235,6 +239,7 @@ __global__ void k_bounds(Grid g, const T* __restrict__ p0, const T* __restrict__
 template <typename T, int ND>
 __global__ void k_antidiff(Grid g, const T* __restrict__ psi, In3<T> Vin, T vscale,
                            const T* __restrict__ G, bool iga, bool tot, bool abs_psi, bool dfl, Out3<T> Vout) {
+  dev::grid_wait();
   // variable-sign option (Sect. 3.1.5): psi enters every psi-fraction as |psi|
   auto ps = [&](long long j) { const T v = psi[j]; return abs_psi ? absv(v) : v; };
   FOR_CELLS(g) {
@@ -374,6 +379,7 @@ template <typename T, bool ABS>
 __global__ void __launch_bounds__(kAx * kAy) k_antidiff3(Grid g, const T* __restrict__ psi, In3<T> Vin,
                                                          T vscale, const T* __restrict__ G, bool iga, bool tot,
                                                          Out3<T> Vout) {
+  dev::grid_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int nP = kPw * kPh, nV = kVw * kVh;
   T* const sP = reinterpret_cast<T*>(smem_raw);  // [kA3P][nP]
@@ -585,6 +591,7 @@ template <typename T>
 __global__ void __launch_bounds__(kAx * kAy) k_p1b3(Grid g, const T* __restrict__ psi, In3<T> V, T vscale,
                                                     const T* __restrict__ G, bool kahan, T* __restrict__ p1,
                                                     T* __restrict__ mx, T* __restrict__ mn) {
+  dev::grid_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int nB = kBw * kBh, nX = kXw * kXh, nH = kHw * kHh;
   T* const sN = reinterpret_cast<T*>(smem_raw);  // [kP1N][nB] psi^n
@@ -757,6 +764,7 @@ __global__ void __launch_bounds__(kAx * kAy) k_corr3(Grid g, const T* __restrict
                                                      const T* __restrict__ mxg, const T* __restrict__ mng,
                                                      const T* __restrict__ R, T dt, bool post, Out3<T> lim,
                                                      T* __restrict__ out) {
+  dev::grid_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* const sm = reinterpret_cast<T*>(smem_raw);
   constexpr int nP = kCPw * kCPh, nV = kCVw * kCVh, nB = kCBw * kCBh;
@@ -996,6 +1004,7 @@ template <typename T, int ND>
 __global__ void k_beta(Grid g, const T* __restrict__ psi, In3<T> V, const T* __restrict__ G, bool unit,
                        const T* __restrict__ mx, const T* __restrict__ mn, T* __restrict__ bu,
                        T* __restrict__ bd) {
+  dev::grid_wait();
   FOR_CELLS(g) {
   const Nbr<ND> nb(g, Coord{{c0_, c1_, c2_}});
   const long long i = nb.i;
@@ -1021,6 +1030,7 @@ __global__ void k_beta(Grid g, const T* __restrict__ psi, In3<T> V, const T* __r
 template <typename T, int ND>
 __global__ void k_limit(Grid g, const T* __restrict__ psi, In3<T> Vu, bool unit,
                         const T* __restrict__ bu, const T* __restrict__ bd, Out3<T> Vout) {
+  dev::grid_wait();
   FOR_CELLS(g) {
   const Nbr<ND> nb(g, Coord{{c0_, c1_, c2_}});
   const long long i = nb.i;
@@ -1211,43 +1221,45 @@ size_t steps1d_smem(long long n) { return static_cast<size_t>(kSteps1dArrays) * 
 
 template <typename T, bool ABS>
 void launch_antidiff3_t(const Grid& g, const T* psi, In3<T> v, T vscale, const T* G, bool iga, bool tot, Out3<T> out,
-                        cudaStream_t st) {
+                        bool chained, cudaStream_t st) {
   static PerDevice<bool> attr;
   attr.get([](int) {
     return cudaFuncSetAttribute(k_antidiff3<T, ABS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 static_cast<int>(antidiff3_smem<T>())) == cudaSuccess;
   });
-  k_antidiff3<T, ABS><<<march3_grid(g), dim3(kAx, kAy), antidiff3_smem<T>(), st>>>(g, psi, v, vscale, G, iga, tot, out);
+  launch_chained(chained, k_antidiff3<T, ABS>, march3_grid(g), dim3(kAx, kAy), antidiff3_smem<T>(), st, g, psi, v, vscale,
+                 G, iga, tot, out);
 }
 
 template <typename T>
 void launch_antidiff3(const Grid& g, const T* psi, In3<T> v, T vscale, const T* G, bool iga, bool tot, bool abs_psi,
-                      Out3<T> out, cudaStream_t st) {
-  if (abs_psi) launch_antidiff3_t<T, true>(g, psi, v, vscale, G, iga, tot, out, st);
-  else launch_antidiff3_t<T, false>(g, psi, v, vscale, G, iga, tot, out, st);
+                      Out3<T> out, bool chained, cudaStream_t st) {
+  if (abs_psi) launch_antidiff3_t<T, true>(g, psi, v, vscale, G, iga, tot, out, chained, st);
+  else launch_antidiff3_t<T, false>(g, psi, v, vscale, G, iga, tot, out, chained, st);
 }
 
 template <typename T>
 void launch_p1b3(const Grid& g, const T* psi, In3<T> v, T vscale, const T* G, bool kahan, T* p1, T* mx, T* mn,
-                 cudaStream_t st) {
+                 bool chained, cudaStream_t st) {
   static PerDevice<bool> attr;
   attr.get([](int) {
     return cudaFuncSetAttribute(k_p1b3<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 static_cast<int>(p1b3_smem<T>())) == cudaSuccess;
   });
-  k_p1b3<T><<<march3_grid(g), dim3(kAx, kAy), p1b3_smem<T>(), st>>>(g, psi, v, vscale, G, kahan, p1, mx, mn);
+  launch_chained(chained, k_p1b3<T>, march3_grid(g), dim3(kAx, kAy), p1b3_smem<T>(), st, g, psi, v, vscale, G, kahan, p1,
+                 mx, mn);
 }
 
 template <typename T>
 void launch_corr3(const Grid& g, const T* psi, In3<T> vu, const T* G, bool unit, bool kahan, const T* mx,
-                  const T* mn, const T* R, T dt, bool post, Out3<T> lim, T* out, cudaStream_t st) {
+                  const T* mn, const T* R, T dt, bool post, Out3<T> lim, T* out, bool chained, cudaStream_t st) {
   static PerDevice<bool> attr;  // the FP64 rings exceed the default 48 KB of dynamic shared memory
   attr.get([](int) {
     return cudaFuncSetAttribute(k_corr3<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 static_cast<int>(corr3_smem<T>())) == cudaSuccess;
   });
-  k_corr3<T><<<march3_grid(g), dim3(kAx, kAy), corr3_smem<T>(), st>>>(g, psi, vu, G, unit, kahan, mx, mn, R, dt,
-                                                                      post, lim, out);
+  launch_chained(chained, k_corr3<T>, march3_grid(g), dim3(kAx, kAy), corr3_smem<T>(), st, g, psi, vu, G, unit, kahan, mx,
+                 mn, R, dt, post, lim, out);
 }
 
 template <typename T, int ND>
@@ -1257,9 +1269,16 @@ cudaError_t staged_nd(const Grid& g, const Opts& o, const StepArgs<T>& a, const 
   const unsigned nb = static_cast<unsigned>((g.N + bs - 1) / bs);
   const int K = o.n_iters;
   const T* G = o.nug ? a.g : nullptr;
+  // every kernel after the first is launched as a dependent of the one before it (launch.cuh), the
+  // first too where that one belongs to the same call
+  bool chain = a.chained;
+  auto go = [&](auto kern, dim3 grid, auto... args) {
+    launch_chained(chain, kern, grid, dim3(bs), 0, st, args...);
+    chain = true;
+  };
   const T* p0 = a.psi_in;
   if (o.rhs_b) {
-    k_pre<T><<<nb, bs, 0, st>>>(g.N, a.psi_in, a.r, a.dt, s.p0);
+    go(k_pre<T>, dim3(nb), g.N, a.psi_in, a.r, a.dt, s.p0);
     p0 = s.p0;
   }
   In3<T> gc{{a.gc[0], a.gc[1], a.gc[2]}};
@@ -1270,17 +1289,18 @@ cudaError_t staged_nd(const Grid& g, const Opts& o, const StepArgs<T>& a, const 
   // recomputes pass 1 on a one-cell halo)
   if (ND == 3 && K >= 2 && o.fct && sizeof(T) == 4 && !o.open) {
     bool done = false;
-    if constexpr (sizeof(T) == 4) done = p1b3_vec(g, p0, gc.p, a.gc_scale, G, o.kahan, s.pa, s.mx, s.mn, st);
-    if (!done) launch_p1b3<T>(g, p0, gc, a.gc_scale, G, o.kahan, s.pa, s.mx, s.mn, st);
+    if constexpr (sizeof(T) == 4) done = p1b3_vec(g, p0, gc.p, a.gc_scale, G, o.kahan, s.pa, s.mx, s.mn, chain, st);
+    if (!done) launch_p1b3<T>(g, p0, gc, a.gc_scale, G, o.kahan, s.pa, s.mx, s.mn, chain, st);
+    chain = true;
   } else {
-    k_donor<T, ND><<<cell_grid(g, bs), bs, 0, st>>>(g, p0, gc, a.gc_scale, false, G, o.kahan, a.r, a.dt,
+    go(k_donor<T, ND>, cell_grid(g, bs), g, p0, gc, a.gc_scale, false, G, o.kahan, a.r, a.dt,
                                       K == 1 && o.rhs_a, dst1);
     if (K == 1) {
       if (dst1 != a.psi_out)
         return cudaMemcpyAsync(a.psi_out, dst1, sizeof(T) * g.N, cudaMemcpyDeviceToDevice, st);
       return cudaGetLastError();
     }
-    if (o.fct) k_bounds<T, ND><<<cell_grid(g, bs), bs, 0, st>>>(g, p0, s.pa, s.mx, s.mn);
+    if (o.fct) go(k_bounds<T, ND>, cell_grid(g, bs), g, p0, s.pa, s.mx, s.mn);
   }
   const T* prev = s.pa;
   In3<T> vprev = gc;
@@ -1291,10 +1311,11 @@ cudaError_t staged_nd(const Grid& g, const Opts& o, const StepArgs<T>& a, const 
     if (ND == 3 && !o.dfl && !o.open) {
       bool done = false;
       if constexpr (sizeof(T) == 4)
-        done = antidiff3_vec(g, prev, vprev.p, vscale, G, o.iga, o.tot, o.abs, vk.p, st);
-      if (!done) launch_antidiff3<T>(g, prev, vprev, vscale, G, o.iga, o.tot, o.abs, vk, st);
+        done = antidiff3_vec(g, prev, vprev.p, vscale, G, o.iga, o.tot, o.abs, vk.p, chain, st);
+      if (!done) launch_antidiff3<T>(g, prev, vprev, vscale, G, o.iga, o.tot, o.abs, vk, chain, st);
+      chain = true;
     } else {
-      k_antidiff<T, ND><<<cell_grid(g, bs), bs, 0, st>>>(g, prev, vprev, vscale, G, o.iga, o.tot, o.abs, o.dfl,
+      go(k_antidiff<T, ND>, cell_grid(g, bs), g, prev, vprev, vscale, G, o.iga, o.tot, o.abs, o.dfl,
                                                          vk);
     }
     In3<T> vuse{{vk.p[0], vk.p[1], vk.p[2]}};
@@ -1308,22 +1329,23 @@ cudaError_t staged_nd(const Grid& g, const Opts& o, const StepArgs<T>& a, const 
       if (k < K) lk = Out3<T>{{lim[0], lim[1], lim[2]}};
       bool done = false;
       if constexpr (sizeof(T) == 4)
-        done = corr3_vec(g, prev, vuse.p, G, o.iga, o.kahan, s.mx, s.mn, k == K && o.rhs_a, lk.p, dst, st);
+        done = corr3_vec(g, prev, vuse.p, G, o.iga, o.kahan, s.mx, s.mn, k == K && o.rhs_a, lk.p, dst, chain, st);
       if (!done)
-        launch_corr3<T>(g, prev, vuse, G, o.iga, o.kahan, s.mx, s.mn, a.r, a.dt, k == K && o.rhs_a, lk, dst, st);
+        launch_corr3<T>(g, prev, vuse, G, o.iga, o.kahan, s.mx, s.mn, a.r, a.dt, k == K && o.rhs_a, lk, dst, chain, st);
+      chain = true;
       prev = dst;
       vprev = In3<T>{{lim[0], lim[1], lim[2]}};
       vscale = T(1);
       continue;
     }
     if (o.fct) {
-      k_beta<T, ND><<<cell_grid(g, bs), bs, 0, st>>>(g, prev, vuse, G, o.iga, s.mx, s.mn, s.bu, s.bd);
+      go(k_beta<T, ND>, cell_grid(g, bs), g, prev, vuse, G, o.iga, s.mx, s.mn, s.bu, s.bd);
       Out3<T> vl{{lim[0], lim[1], lim[2]}};
-      k_limit<T, ND><<<cell_grid(g, bs), bs, 0, st>>>(g, prev, vuse, o.iga, s.bu, s.bd, vl);
+      go(k_limit<T, ND>, cell_grid(g, bs), g, prev, vuse, o.iga, s.bu, s.bd, vl);
       vuse = In3<T>{{lim[0], lim[1], lim[2]}};
     }
     T* dst = (k == K) ? a.psi_out : (prev == s.pa ? s.pb : s.pa);
-    k_donor<T, ND><<<cell_grid(g, bs), bs, 0, st>>>(g, prev, vuse, T(1), o.iga, G, o.kahan, a.r, a.dt,
+    go(k_donor<T, ND>, cell_grid(g, bs), g, prev, vuse, T(1), o.iga, G, o.kahan, a.r, a.dt,
                                       k == K && o.rhs_a, dst);
     prev = dst;
     vprev = vuse;
@@ -1342,7 +1364,7 @@ cudaError_t tape_nd(const Grid& g, const Opts& o, const T* const* gc, const T* G
     k_donor<T, ND><<<cell_grid(g, bs), bs, 0, st>>>(g, tp.psi[0], v1, T(1), false, G, o.kahan, nullptr, T(0), false, psi_next);
   if (K >= 2) {
     if (ND == 3 && o.fct && sizeof(T) == 4) {
-      launch_p1b3<T>(g, tp.psi[0], v1, T(1), G, o.kahan, levels[1], tp.mx, tp.mn, st);
+      launch_p1b3<T>(g, tp.psi[0], v1, T(1), G, o.kahan, levels[1], tp.mx, tp.mn, false, st);
     } else {
       k_donor<T, ND><<<cell_grid(g, bs), bs, 0, st>>>(g, tp.psi[0], v1, T(1), false, G, o.kahan, nullptr, T(0), false,
                                                       levels[1]);
@@ -1353,7 +1375,7 @@ cudaError_t tape_nd(const Grid& g, const Opts& o, const T* const* gc, const T* G
     In3<T> vprev{{tp.vh[k - 1][0], tp.vh[k - 1][1], tp.vh[k - 1][2]}};
     Out3<T> vk{{tp.v[k][0], tp.v[k][1], tp.v[k][2]}};
     if (ND == 3 && !o.dfl) {  // the z-march leaves the divergent-flow term to the generic kernel
-      launch_antidiff3<T>(g, tp.psi[k - 1], vprev, T(1), G, o.iga, o.tot, o.abs, vk, st);
+      launch_antidiff3<T>(g, tp.psi[k - 1], vprev, T(1), G, o.iga, o.tot, o.abs, vk, false, st);
     } else {
       k_antidiff<T, ND><<<cell_grid(g, bs), bs, 0, st>>>(g, tp.psi[k - 1], vprev, T(1), G, o.iga, o.tot, o.abs,
                                                          o.dfl, vk);

@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 
 #include "internal.h"
+#include "launch.cuh"
 
 namespace mpd {
 namespace {
@@ -37,6 +38,7 @@ __device__ __forceinline__ long long nb(const Grid& g, const int (&c)[3], long l
 template <typename T>
 __global__ void k_vip_cells(long long n, int nd, const T* __restrict__ state, T* __restrict__ uprev,
                             T* __restrict__ ext, bool first, T eps) {
+  dev::grid_wait();
   for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
        i += static_cast<long long>(gridDim.x) * blockDim.x) {
     const T h = state[i];
@@ -51,6 +53,7 @@ __global__ void k_vip_cells(long long n, int nd, const T* __restrict__ state, T*
 
 template <typename T>
 __global__ void k_vip_faces(Grid g, const T* __restrict__ ext, T* __restrict__ adv, T courant) {
+  dev::grid_wait();
   const long long n = g.N;
   for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
        i += static_cast<long long>(gridDim.x) * blockDim.x) {
@@ -66,6 +69,7 @@ __global__ void k_vip_faces(Grid g, const T* __restrict__ ext, T* __restrict__ a
 
 template <typename T>
 __global__ void k_sw_force(Grid g, T* __restrict__ state, T half_dt, T inv2dx) {
+  dev::grid_wait();
   const long long n = g.N;
   for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
        i += static_cast<long long>(gridDim.x) * blockDim.x) {
@@ -89,23 +93,24 @@ unsigned blocks_of(long long n) {
 
 template <typename T>
 cudaError_t vip_advector(const Grid& g, const T* state, T* uprev, T* ext, T* adv, bool first, T eps, T courant,
-                         cudaStream_t st) {
-  k_vip_cells<T><<<blocks_of(g.N), 256, 0, st>>>(g.N, g.nd, state, uprev, ext, first, eps);
-  k_vip_faces<T><<<blocks_of(g.N), 256, 0, st>>>(g, ext, adv, courant);
+                         bool chained, cudaStream_t st) {
+  const dim3 blocks(blocks_of(g.N));
+  launch_chained(chained, k_vip_cells<T>, blocks, dim3(256), 0, st, g.N, g.nd, state, uprev, ext, first, eps);
+  launch_chained(true, k_vip_faces<T>, blocks, dim3(256), 0, st, g, ext, adv, courant);
   return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t sw_force(const Grid& g, T* state, T half_dt, T dx, cudaStream_t st) {
-  k_sw_force<T><<<blocks_of(g.N), 256, 0, st>>>(g, state, half_dt, T(1) / (T(2) * dx));
+cudaError_t sw_force(const Grid& g, T* state, T half_dt, T dx, bool chained, cudaStream_t st) {
+  launch_chained(chained, k_sw_force<T>, dim3(blocks_of(g.N)), dim3(256), 0, st, g, state, half_dt, T(1) / (T(2) * dx));
   return cudaGetLastError();
 }
 
 template cudaError_t vip_advector<float>(const Grid&, const float*, float*, float*, float*, bool, float, float,
-                                         cudaStream_t);
+                                         bool, cudaStream_t);
 template cudaError_t vip_advector<double>(const Grid&, const double*, double*, double*, double*, bool, double,
-                                          double, cudaStream_t);
-template cudaError_t sw_force<float>(const Grid&, float*, float, float, cudaStream_t);
-template cudaError_t sw_force<double>(const Grid&, double*, double, double, cudaStream_t);
+                                          double, bool, cudaStream_t);
+template cudaError_t sw_force<float>(const Grid&, float*, float, float, bool, cudaStream_t);
+template cudaError_t sw_force<double>(const Grid&, double*, double, double, bool, cudaStream_t);
 
 }  // namespace mpd
