@@ -343,9 +343,9 @@ __global__ void __launch_bounds__(W * 32, 2) k_band2d(const BandParams<T> p) {
         const T A = IGA ? d * T(0.5) : ratio(d, S0[c]);
         const T Tt = right_of(S0, c, S0R), Bt = left_of(S0, c, S0L);
         const T B = IGA ? (Tt - Bt) * T(0.25) : ratio(Tt - Bt, Tt + Bt);
-        const T Vq = T(0.25) * (PV1[c] + left_of(PV1, c, PV1L));
+        const T Vs = PV1[c] + left_of(PV1, c, PV1L);  // four times the mean transverse advector
         const T rGb = NUG ? fdiv(T(1), Gb) : T(1);
-        const T out = (absv(V) - V * V * rGb) * A - T(0.5) * V * Vq * rGb * B;
+        const T out = (absv(V) - V * V * rGb) * A - T(0.125) * V * Vs * rGb * B;
         u0n[c] = IGA ? out : flux(q_c[c], p1_c[c], out);
         na0[c] = out;
         pvp[c] = v0_m[c] + right_of(v0_m, c, v0R);
@@ -372,9 +372,9 @@ __global__ void __launch_bounds__(W * 32, 2) k_band2d(const BandParams<T> p) {
           const T A = IGA ? (q1 - q0) * T(0.5) : ratio(q1 - q0, Sc);
           const T B = IGA ? (Sp - Sm) * T(0.25) : ratio(Sp - Sm, Sp + Sm);
           const T pvm = w0_m[c] + right_of(w0_m, c, w0R);
-          const T Vq = T(0.25) * (pvp[c] + pvm);
+          const T Vs = pvp[c] + pvm;
           const T rGb = NUG ? fdiv(T(1), Gb) : T(1);
-          const T out = (absv(V) - V * V * rGb) * A - T(0.5) * V * Vq * rGb * B;
+          const T out = (absv(V) - V * V * rGb) * A - T(0.125) * V * Vs * rGb * B;
           u1n[c] = IGA ? out : flux(q0, q1, out);
           na1[c] = out;
         }
@@ -413,11 +413,8 @@ __global__ void __launch_bounds__(W * 32, 2) k_band2d(const BandParams<T> p) {
         for (int c = 0; c < NC; ++c) {
           const T Fm0 = u0m[c], Fp0 = u0n[c];
           const T Fp1 = u1n[c], Fm1 = left_of(u1n, c, u1L);
-          // [x]- = x - [x]+ and [x]+ = x - [x]- hold exactly in floating point, so the
-          // outflow sum reuses the inflow sum's four extrema (adds instead of min/max)
-          const T pFm0 = posp(Fm0), nFp0 = negp(Fp0), pFm1 = posp(Fm1), nFp1 = negp(Fp1);
-          const T in = (pFm0 - nFp0) + (pFm1 - nFp1);
-          const T ou = ((Fp0 - nFp0) - (Fm0 - pFm0)) + ((Fp1 - nFp1) - (Fm1 - pFm1));
+          T in, ou;
+          flow_sums(Fm0, Fp0, Fm1, Fp1, in, ou);
           const T Gi = NUG ? g_b[c] : T(1);
           const T q = q_c[c];
           // mx - q and q - mn are never negative (q is one of the candidates); min(1, x / |s|)

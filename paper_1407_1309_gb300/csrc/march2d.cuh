@@ -271,9 +271,9 @@ __device__ __forceinline__ void march_tile(const F2Params<T>& p, const int strip
         const T A = IGA ? d * T(0.5) : ratio(d, S0[c]);
         const T Tt = right_of(S0, c, S0R), Bt = left_of(S0, c, S0L);
         const T B = IGA ? (Tt - Bt) * T(0.25) : ratio(Tt - Bt, Tt + Bt);
-        const T Vq = T(0.25) * (PV1[c] + left_of(PV1, c, PV1L));
+        const T Vs = PV1[c] + left_of(PV1, c, PV1L);  // four times the mean transverse advector
         const T rGb = NUG ? fdiv(T(1), Gb) : T(1);
-        T out = (absv(V) - V * V * rGb) * A - T(0.5) * V * Vq * rGb * B;
+        T out = (absv(V) - V * V * rGb) * A - T(0.125) * V * Vs * rGb * B;
         if (DFL) out = out - T(0.25) * V * (dv[0][c] + dv[1][c]) * rGb;
         na0[c] = out;
         nu0[c] = IGA ? out : flux(p1[2][c], p1[3][c], out);
@@ -303,9 +303,9 @@ __device__ __forceinline__ void march_tile(const F2Params<T>& p, const int strip
         const T q0 = p1[2][c], q1 = right_of(p1[2], c, p1r[1]);
         const T A = IGA ? (q1 - q0) * T(0.5) : ratio(fr(q1) - fr(q0), Sc[c]);
         const T B = IGA ? (Sp[c] - Sm[c]) * T(0.25) : ratio(Sp[c] - Sm[c], Sp[c] + Sm[c]);
-        const T Vq = T(0.25) * (pv0[1][c] + pv0[0][c]);
+        const T Vs = pv0[1][c] + pv0[0][c];
         const T rGb = NUG ? fdiv(T(1), Gb) : T(1);
-        T out = (absv(V) - V * V * rGb) * A - T(0.5) * V * Vq * rGb * B;
+        T out = (absv(V) - V * V * rGb) * A - T(0.125) * V * Vs * rGb * B;
         if (DFL) out = out - T(0.25) * V * (dv[0][c] + right_of(dv[0], c, dvR)) * rGb;
         na1[c] = out;
         nu1[c] = IGA ? out : flux(q0, q1, out);
@@ -325,11 +325,8 @@ __device__ __forceinline__ void march_tile(const F2Params<T>& p, const int strip
           const T mn = min3(min3(lo[1][c], lo[0][c], lo[2][c]), left_of(lo[1], c, lL), right_of(lo[1], c, lR));
           const T Fm0 = u0[0][c], Fp0 = u0[1][c];
           const T Fp1 = u1[1][c], Fm1 = left_of(u1[1], c, u1L);
-          // [x]- = x - [x]+ and [x]+ = x - [x]- hold exactly in floating point, so the
-          // outflow sum reuses the inflow sum's four extrema (adds instead of min/max)
-          const T pFm0 = posp(Fm0), nFp0 = negp(Fp0), pFm1 = posp(Fm1), nFp1 = negp(Fp1);
-          const T in = (pFm0 - nFp0) + (pFm1 - nFp1);
-          const T ou = ((Fp0 - nFp0) - (Fm0 - pFm0)) + ((Fp1 - nFp1) - (Fm1 - pFm1));
+          T in, ou;
+          flow_sums(Fm0, Fp0, Fm1, Fp1, in, ou);
           const T Gi = NUG ? gg[1][c] : T(1);
           const T q = p1[2][c];
           // mx - q and q - mn are never negative (q is one of the candidates); min(1, x / |s|)

@@ -13,7 +13,9 @@
 // shallow-water system) share a launch, one grid layer each.
 //
 // Measured: a shallow-water step of three 320^2 FP64 fields with open edges, |psi|, limiter and
-// divergent-flow term 218 -> 110 us (the FP64 pipe's floor is about 70 us).
+// divergent-flow term 218 us staged, 96 here with its source kernels (the FP64 pipe's floor is about
+// 65 us); sign tests in place of products, the divergence once per cell and 32-row tiles took it
+// there from 108.
 //
 // Open edges (Sect. 2.4): only cells of the field are computed; a neighbour beyond an open edge is
 // the edge cell, a face beyond it the adjacent interior face (offset clamping, in the tiles that
@@ -32,8 +34,7 @@ namespace {
 using namespace dev;
 
 constexpr int kThreadsT = 256;
-constexpr int kCols = 32;                                       // tile columns
-template <typename T> constexpr int tile_rows() { return sizeof(T) == 4 ? 32 : 16; }
+constexpr int kCols = 32;  // tile columns; rows: 32, or 16 (FP64 fields with too few tiles of 32)
 
 template <typename T>
 struct TileParams {
@@ -97,9 +98,8 @@ __device__ __forceinline__ bool sum_counts(double x) { return gt0(x) && divisibl
 __device__ __forceinline__ bool zero(float x) { return x == 0.0f; }
 __device__ __forceinline__ bool zero(double x) { return !nonzero(x); }
 
-template <typename T, bool FCT, bool IGA, bool NUG>
+template <typename T, int kRows, bool FCT, bool IGA, bool NUG>
 __global__ void __launch_bounds__(kThreadsT, 2) k_tile2d(const TileParams<T> p) {
-  constexpr int kRows = tile_rows<T>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int H = p.H, L = kCols + 2 * H, A = (kRows + 2 * H) * L;
   T* cur = reinterpret_cast<T*>(smem_raw);  // psi^(k-1)
@@ -113,6 +113,7 @@ __global__ void __launch_bounds__(kThreadsT, 2) k_tile2d(const TileParams<T> p) 
   T* const MX = BD + A;                     // bounds, with more than two passes and the limiter
   T* const MN = MX + A;
   T* const Gs = FCT ? (p.K > 2 ? MN + A : MX) : BU;
+  T* const DV = Gs + (NUG ? A : 0);         // the advector's difference across the cell (divergent flow)
   const int R0 = static_cast<int>(blockIdx.y) * kRows, Q0 = static_cast<int>(blockIdx.x) * kCols;
   const int x0 = R0 - H, y0 = Q0 - H;  // field row and column of the tile array's corner
   const T* const psi = p.psi + blockIdx.z * p.field;
@@ -164,7 +165,9 @@ __global__ void __launch_bounds__(kThreadsT, 2) k_tile2d(const TileParams<T> p) 
     over(H - m, H + kRows + m, H - m, H + kCols + m, [&](int r, int c) {
       if (!inside(r, c)) return;
       const int i = r * L + c;
-      nxt[i] = donor(cur, C0, C1, i, offs(e0, x0 + r, p.n0, L), offs(e1, y0 + c, p.n1, 1), false);
+      const Off a = offs(e0, x0 + r, p.n0, L), b = offs(e1, y0 + c, p.n1, 1);
+      nxt[i] = donor(cur, C0, C1, i, a, b, false);
+      if (p.dfl) DV[i] = (C0[i + a.f0] - C0[i + a.fm]) + (C1[i + b.f0] - C1[i + b.fm]);
     });
   }
   __syncthreads();
@@ -192,7 +195,7 @@ __global__ void __launch_bounds__(kThreadsT, 2) k_tile2d(const TileParams<T> p) 
         const T Av = IGA ? (f1 - f0) * T(0.5) : ratio(f1 - f0, f0 + f1);
         T o = (absv(V) - V * V * rGb) * Av;
         const T q0 = Q[i + q.f0], q1 = Q[ip + q.f0], q2 = Q[i + q.fm], q3 = Q[ip + q.fm];
-        const T Vq = T(0.25) * ((q0 + q1) + (q2 + q3));
+        const T Vs = (q0 + q1) + (q2 + q3);  // four times the mean transverse advector
         const T x = fr(cur[i + q.p1]), y = fr(cur[ip + q.p1]), z = fr(cur[i + q.m1]), w = fr(cur[ip + q.m1]);
         const T Tp = x + y, Bt = z + w;
         T B, D2 = T(0);
@@ -204,19 +207,15 @@ __global__ void __launch_bounds__(kThreadsT, 2) k_tile2d(const TileParams<T> p) 
         } else {
           B = ratio(Tp - Bt, Tp + Bt);
         }
-        o = o - T(0.5) * V * Vq * rGb * B;
+        o = o - T(0.125) * V * Vs * rGb * B;
         if (p.tot) {
           const T fm = fr(cur[i + d.m1]), f2 = fr(cur[i + d.p2]);
           const T num = ((f2 - f1) - f0) + fm;
           const T Dd = IGA ? num * T(0.25) : ratio(num, ((f2 + f1) + f0) + fm);
           o = o + ((T(3) * V * absv(V)) * rGb - (T(2) * V * V * V) * (rGb * rGb) - V) * T(1.0 / 3.0) * Dd;
-          o = o + absv(V) * Vq * rGb * (T(1) - T(2) * absv(V) * rGb) * D2;
+          o = o + absv(V) * (T(0.25) * Vs) * rGb * (T(1) - T(2) * absv(V) * rGb) * D2;
         }
-        if (p.dfl) {
-          const T along = (D[i + d.f0] - D[i + d.fm]) + (D[i + d.fp] - D[i + d.f0]);
-          const T across = (q0 - q2) + (q1 - q3);
-          o = o - T(0.25) * V * (along + across) * rGb;
-        }
+        if (p.dfl) o = o - T(0.25) * V * (DV[i] + DV[ip]) * rGb;
         return o;
       };
       if (c >= lo) W0[i] = face(a, b, C0, C1);
@@ -244,8 +243,8 @@ __global__ void __launch_bounds__(kThreadsT, 2) k_tile2d(const TileParams<T> p) 
         const T v0p = W0[i + a.f0], v0m = W0[i + a.fm], v1p = W1[i + b.f0], v1m = W1[i + b.fm];
         const T Fp0 = IGA ? v0p : flux(q, qu, v0p), Fm0 = IGA ? v0m : flux(qd, q, v0m);
         const T Fp1 = IGA ? v1p : flux(q, qr, v1p), Fm1 = IGA ? v1m : flux(ql, q, v1m);
-        const T in = (posp(Fm0) - negp(Fp0)) + (posp(Fm1) - negp(Fp1));
-        const T ou = (posp(Fp0) - negp(Fm0)) + (posp(Fp1) - negp(Fm1));
+        T in, ou;
+        flow_sums(Fm0, Fp0, Fm1, Fp1, in, ou);
         T up = posp(mx - q), dn = posp(q - mn);
         if (NUG) { up = Gs[i] * up; dn = Gs[i] * dn; }
         BU[i] = sum_counts(in) ? fdiv(up, in) : T(1);
@@ -258,9 +257,10 @@ __global__ void __launch_bounds__(kThreadsT, 2) k_tile2d(const TileParams<T> p) 
         if (!inside(r, c)) return;
         const int i = r * L + c;
         auto limit = [&](T* W, int ip) {
-          const T V = W[i];
-          const T F = IGA ? V : flux(cur[i], cur[ip], V);
-          const bool right = gt0(F) || (zero(F) && gt0(V));
+          // the unlimited flux V up goes right where V and the upwind value have the same sign, or,
+          // where it is zero, where V > 0 (signs alone: no product on the FP64 pipe)
+          const T V = W[i], up = gt0(V) ? cur[i] : cur[ip];
+          const bool right = IGA || zero(up) ? gt0(V) : !zero(V) && gt0(V) == gt0(up);
           W[i] = V * min3(T(1), right ? BD[i] : BU[i], right ? BU[ip] : BD[ip]);
         };
         // an open edge's last stored face is not one of its cells' faces
@@ -289,28 +289,54 @@ __global__ void __launch_bounds__(kThreadsT, 2) k_tile2d(const TileParams<T> p) 
       T* t = cur; cur = nxt; nxt = t;
       t = C0; C0 = W0; W0 = t;
       t = C1; C1 = W1; W1 = t;
+      if (p.dfl) {  // of the advector that drives the next pass, on the cells of its faces
+        const int w = m - p.reach + (FCT ? 2 : 1);
+        over(H - w, H + kRows + w, H - w, H + kCols + w, [&](int r, int c) {
+          if (!inside(r, c)) return;
+          const int i = r * L + c;
+          const Off a = offs(e0, x0 + r, p.n0, L), b = offs(e1, y0 + c, p.n1, 1);
+          DV[i] = (C0[i + a.f0] - C0[i + a.fm]) + (C1[i + b.f0] - C1[i + b.fm]);
+        });
+        __syncthreads();
+      }
     }
   }
 }
 
-template <typename T, bool FCT, bool IGA, bool NUG>
-int launch_tile(const TileParams<T>& p, int fields, cudaStream_t st) {
-  constexpr int kRows = tile_rows<T>();
-  const size_t arrays = 6 + (FCT ? 2 + (p.K > 2 ? 2 : 0) : 0) + (NUG ? 1 : 0);
+template <typename T, int kRows, bool FCT, bool IGA, bool NUG>
+int launch_rows(const TileParams<T>& p, int fields, cudaStream_t st) {
+  const size_t arrays = 6 + (FCT ? 2 + (p.K > 2 ? 2 : 0) : 0) + (NUG ? 1 : 0) + (p.dfl ? 1 : 0);
   const size_t smem = sizeof(T) * arrays * (kRows + 2 * p.H) * (kCols + 2 * p.H);
   static PerDevice<int> most_of;
   const int most = most_of.get([](int dev) {
     int m = 0;
     cudaDeviceGetAttribute(&m, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    cudaFuncSetAttribute(k_tile2d<T, FCT, IGA, NUG>, cudaFuncAttributeMaxDynamicSharedMemorySize, m);
+    cudaFuncSetAttribute(k_tile2d<T, kRows, FCT, IGA, NUG>, cudaFuncAttributeMaxDynamicSharedMemorySize, m);
     return m;
   });
   const long long ty = (p.n0 + kRows - 1) / kRows;
   if (smem > static_cast<size_t>(most) || ty > 65535) return MPDATA_EUNSUPPORTED;
   const dim3 grid(static_cast<unsigned>((p.n1 + kCols - 1) / kCols), static_cast<unsigned>(ty),
                   static_cast<unsigned>(fields));
-  launch_chained(p.chained, k_tile2d<T, FCT, IGA, NUG>, grid, dim3(kThreadsT), smem, st, p);
+  launch_chained(p.chained, k_tile2d<T, kRows, FCT, IGA, NUG>, grid, dim3(kThreadsT), smem, st, p);
   return cudaGetLastError() == cudaSuccess ? MPDATA_OK : MPDATA_ECUDA;
+}
+
+template <typename T, bool FCT, bool IGA, bool NUG>
+int launch_tile(const TileParams<T>& p, int fields, cudaStream_t st) {
+  if constexpr (sizeof(T) == 8) {
+    // 32 rows repeat less of the halo's arithmetic (1.13x instead of 1.2x with H = 3), 16 rows feed
+    // more SMs: the taller tile where it leaves nearly every SM two blocks and its shared memory
+    // fits
+    const long long tall = static_cast<long long>(fields) * ((p.n0 + 31) / 32) * ((p.n1 + kCols - 1) / kCols);
+    if (tall >= 280) {
+      const int rc = launch_rows<T, 32, FCT, IGA, NUG>(p, fields, st);
+      if (rc != MPDATA_EUNSUPPORTED) return rc;
+    }
+    return launch_rows<T, 16, FCT, IGA, NUG>(p, fields, st);
+  } else {
+    return launch_rows<T, 32, FCT, IGA, NUG>(p, fields, st);
+  }
 }
 
 }  // namespace

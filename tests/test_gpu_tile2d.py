@@ -56,3 +56,23 @@ def test_tile_step_matches_oracle(dtype, shape, name, edges):
         assert np.abs(got - ref).max() <= 1e-12 * np.abs(ref).max()
     else:
         assert np.linalg.norm(got - ref) <= 1e-5 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("edges", ["periodic", "open"])
+@pytest.mark.parametrize("name", ["abs_dfl_fct", "dfl_tot3_fct"])
+def test_tall_fp64_tiles_match_oracle(name, edges):
+    """FP64 fields with enough tiles for the 32-row form (18 x 17 tiles, the last ones partial)."""
+    n_iters, opts = OPTS[name]
+    opts = opts | OPEN[edges]
+    shape = (563, 530)
+    rng = np.random.default_rng(8)
+    psi = smooth_positive(shape, rng) - (1.2 if opts & capi.ABS else 0.0)
+    gc = [0.15 * rng.uniform(-1, 1, size=shape) for _ in range(2)]
+    t = lambda a: torch.tensor(a, dtype=torch.float64, device=DEV)
+    oracle.set_threads(0)
+    ref = oracle.step(psi, gc, n_iters=n_iters, opts=int(opts), n_steps=2)
+    with Mpdata(shape, dtype=torch.float64, n_iters=n_iters, opts=opts) as m:
+        out = t(psi)
+        m.advance(t(psi), out, [t(v) for v in gc], n_steps=2)
+        torch.cuda.synchronize()
+        assert np.abs(out.cpu().numpy() - ref).max() <= 1e-12 * np.abs(ref).max()
