@@ -470,10 +470,11 @@ inline bool al(const void* q, size_t a) { return q == nullptr || (reinterpret_ca
 // Tile height of the FP32 warp march and the time it should take.  Every warp of a tile height ty
 // marches ty + 6 rows; with k blocks on the fullest SM one row of all of them takes it c(k)
 // microseconds, more than k times one block's share only while few warps leave the issue slots idle
-// (c measured on fields of 256^2 .. 4096^2: one block takes almost as long as two).  The
-// height is the smallest that keeps the fullest SM at k blocks, for the k of least time.  Against
-// the earlier list of heights (the tallest with 7.5 warps per SM): 4096^2 102 -> 96 us (121 rows
-// instead of 64), 2000 x 500 13.9 -> 10.8 us (with lanes of 2).
+// (c measured on fields of 256^2 .. 4096^2: one block takes almost as long as two; three of the
+// plain march with lanes of 4 fit an SM at once).  The height is the smallest that keeps the fullest
+// SM at k blocks, for the k of least time.  Against the earlier list of heights (the tallest with
+// 7.5 warps per SM): 4096^2 102 -> 89 us (79 rows instead of 64), 2000 x 500 13.9 -> 10.8 us (with
+// lanes of 2).
 struct MarchRows {
   int ty;
   float us;
@@ -481,7 +482,7 @@ struct MarchRows {
 template <int NC>
 inline MarchRows march_rows(int n0, int n1, bool comp) {
   static_assert(NC == 4 || NC == 2, "lanes of 4 or 2 columns");
-  static const float plain4[4] = {0.55f, 0.70f, 1.05f, 1.42f}, plain2[4] = {0.38f, 0.455f, 0.59f, 0.74f};
+  static const float plain4[4] = {0.55f, 0.73f, 1.00f, 1.44f}, plain2[4] = {0.38f, 0.455f, 0.59f, 0.74f};
   static const float comp4[4] = {0.93f, 0.97f, 1.37f, 1.83f}, comp2[4] = {0.53f, 0.58f, 0.76f, 0.97f};
   const float* c = NC == 4 ? (comp ? comp4 : plain4) : (comp ? comp2 : plain2);
   const long long strips = (n1 + stride<NC>() - 1) / stride<NC>();
@@ -495,7 +496,7 @@ inline MarchRows march_rows(int n0, int n1, bool comp) {
     if (ty < 4) ty = 4;
     const long long blocks = (strips * ((n0 + ty - 1) / ty) + kWarps - 1) / kWarps;
     const long long full = (blocks + kSms - 1) / kSms;
-    const float us = static_cast<float>(ty + 6) * (full <= 4 ? c[full - 1] : 0.25f * c[3] * static_cast<float>(full));
+    const float us = static_cast<float>(ty + 6) * (full <= 4 ? c[full - 1] : c[2] / 3.0f * static_cast<float>(full));
     if (!any || us < best.us) best = {static_cast<int>(ty), us};
     any = true;
   }
