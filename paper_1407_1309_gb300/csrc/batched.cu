@@ -15,9 +15,31 @@ namespace {
 struct TableHolder {
   BatchTable tab{};
   int nc = 0;
+  int rows = 0, kernel = 0;  // the MPDATA_TUNE_TILE_ROWS and MPDATA_TUNE_KERNEL it was built for
 };
 
-constexpr int kDefaultBatchRows = 32;
+// Tile height of an ensemble and the time a step should take (microseconds).  The tiles are dealt out
+// in turn to the warps of a persistent grid of up to `most` blocks of 4 per SM, each marching its
+// rows and a 6-row ramp: a warp's share is the rows of all tiles over the warps, plus on average half
+// a tile that ends after the others.  With k blocks on the fullest SM a row takes them row_us[k - 1].
+struct BatchRows {
+  int ty;
+  double us;
+};
+BatchRows batch_rows(const Grid* grids, int nf, int strip, int most, const double* row_us) {
+  BatchRows best{32, -1.0};
+  for (int ty : {8, 12, 16, 24, 32, 48, 64, 96, 128}) {
+    long long tiles = 0;
+    for (int f = 0; f < nf; ++f)
+      tiles += static_cast<long long>((grids[f].n[2] + strip - 1) / strip) * ((grids[f].n[1] + ty - 1) / ty);
+    const long long one = 152 * 4;  // warps of one block per SM
+    const long long k = tiles > one * most ? most : (tiles + one - 1) / one;
+    const double share = tiles > one * k ? static_cast<double>(tiles) / static_cast<double>(one * k) + 0.5 : 1.0;
+    const double us = row_us[k - 1] * share * (ty + 6);
+    if (best.us < 0.0 || us < best.us) best = {ty, us};
+  }
+  return best;
+}
 
 }  // namespace
 
@@ -36,12 +58,25 @@ template <typename T>
 int batched_step(mpdata_s* h, const T* psi_in, T* psi_out, const T* const* gc, const T* g, const T* r, T dt,
                  T gc_scale, bool chained, const Opts& o) {
   if (handle_nd(h) != 2 || o.n_iters != 2 || o.tot || o.abs || o.dfl || o.open) return MPDATA_EUNSUPPORTED;
-  // lanes of 2 columns for FP32 when the handle asks for them (MPDATA_TUNE_KERNEL = 3)
-  const int nc = (o.kernel == 3 && sizeof(T) == 4) ? 2 : fused_batched_columns<T>();
-  const int ty = o.tile_rows > 0 ? o.tile_rows : kDefaultBatchRows;
   void** slot = handle_batch(h);
   auto* th = static_cast<TableHolder*>(*slot);
-  if (th == nullptr || th->tab.ty != ty || th->nc != nc) {
+  if (th == nullptr || th->rows != o.tile_rows || th->kernel != o.kernel) {
+    // FP32 lanes of 4 columns (two blocks fit an SM) or of 2 (four), whichever should be faster: the
+    // narrower strips pad less and give a small ensemble more warps (100 fields of 60^2 .. 300^2: 53 ->
+    // 36 us per step, 20 of 40^2 .. 120^2: 25 -> 8; 512 fields of 64^2 .. 512^2 with lanes of 4: 389,
+    // with lanes of 2: 400).  MPDATA_TUNE_KERNEL = 3 asks for lanes of 2.
+    constexpr int wide = sizeof(T) == 4 ? 4 : 2;
+    static const double us4[2] = {0.55, 0.73}, us2[4] = {0.38, 0.455, 0.59, 0.74};
+    const BatchRows by_wide = batch_rows(handle_grids(h), handle_fields(h), fused_strip_stride(wide), 2, us4);
+    int nc = wide, ty = by_wide.ty;
+    if (sizeof(T) == 4 && (o.kernel == 3 || (o.kernel == 0 && o.tile_rows == 0))) {
+      const BatchRows by_2 = batch_rows(handle_grids(h), handle_fields(h), fused_strip_stride(2), 4, us2);
+      if (o.kernel == 3 || by_2.us < by_wide.us) {
+        nc = 2;
+        ty = by_2.ty;
+      }
+    }
+    if (o.tile_rows > 0) ty = o.tile_rows;
     batched_free(h);
     const int nf = handle_fields(h);
     const Grid* grids = handle_grids(h);
@@ -63,6 +98,8 @@ int batched_step(mpdata_s* h, const T* psi_in, T* psi_out, const T* const* gc, c
     }
     th = new TableHolder;
     th->nc = nc;
+    th->rows = o.tile_rows;
+    th->kernel = o.kernel;
     th->tab.ty = ty;
     th->tab.n_items = static_cast<int>(item_field.size());
     if (cudaMalloc(&th->tab.fields, sizeof(BatchField) * nf) != cudaSuccess ||
