@@ -457,10 +457,15 @@ void launch_band(BandParams<T> p, int tile_rows, cudaStream_t st) {
   });
   if (tile_rows > 0) {
     p.H = tile_rows;
-  } else {  // one band per resident block: as few, tall bands as fill the GPU once
+  } else {
+    // Small fields: bands of W - 6 = 2 rows, one chunk with the halo, where all of them are resident at
+    // once (59 x 61 FP32 4.0 -> 2.9 us per step, FP64 19.1 -> 9.6).  Else one band per resident block,
+    // as few, tall bands as fill the GPU once, at least 8 rows.
+    constexpr int kShort = W - 6;
     const int bands = slots / p.strips > 1 ? slots / p.strips : 1;
     p.H = (p.n0 + bands - 1) / bands;
-    if (p.H < 8) p.H = 8;
+    if (p.H <= kShort) p.H = kShort;
+    else if (p.H < 8) p.H = 8;
   }
   const long long blocks = static_cast<long long>(p.strips) * ((p.n0 + p.H - 1) / p.H);
   const size_t smem = band_smem<T>(3 + (NUG ? 1 : 0) + (p.rhs_b ? 1 : 0), FCT);
