@@ -135,9 +135,9 @@ def measured_peaks():
 
 
 KERNEL_NAMES = {1: "k_fused2d", 2: "k_band2d", 3: "k_fused2d_nc2"}
-KERNEL_SOURCES = {"k_fused2d": ("fused2d.cu", "stencil2d.cuh"), "k_band2d": ("band2d.cu", "stencil2d.cuh"),
-                  "k_fused2d_comp": ("fused2d.cu", "stencil2d.cuh"), "k_fused2d_nc2": ("fused2d.cu", "stencil2d.cuh"),
-                  "k_fused2d_comp_nc2": ("fused2d.cu", "stencil2d.cuh")}
+_WARP_MARCH = ("fused2d.cu", "march2d.cuh", "stencil2d.cuh")
+KERNEL_SOURCES = {"k_fused2d": _WARP_MARCH, "k_band2d": ("band2d.cu", "stencil2d.cuh"), "k_fused2d_comp": _WARP_MARCH,
+                  "k_fused2d_nc2": _WARP_MARCH, "k_fused2d_comp_nc2": _WARP_MARCH}
 
 
 def kernel_sources_sha256(kernel):
@@ -202,17 +202,16 @@ def alu_roofline(cells, seconds_per_step, kernel, n, dtype, sm_max_mhz, sm_count
 
 # FP64 arithmetic per cell-step (adds, multiplies and fused multiply-adds, one each: the work of
 # the FP64 pipe, in the unit of the measured FMA rate; comparisons and selections not counted, a
-# division being the Newton-Raphson division with remainder correction, 7):
-#   2D (n_iters = 2, FCT, G = 1), 94, counted from the formulas: pass 1 6 (two face fluxes, three
-#   flux differences, the update), pseudo-velocities 29 per face (A and B 9 each, V_q 3, the
-#   combination 7, the flux 1), FCT 24 (in/out sums 8, two factors 8 each), limited fluxes 2,
-#   pass 2 4 (the 2D kernels execute 118 per cell-step at 1024^2, their recomputed halo included);
-#   3D (n_iters = 3 + tot + FCT + G), 992, counted by ncu as the DADD + DMUL + DFMA instructions of
-#   one step of the staged FP64 kernels at 128^3 (no recomputed halo): pass 1 46, the bounds 0,
-#   per corrective pass 473 (pseudo-advector with the cross and third-order terms 376, factors 42,
-#   limiter 9, donor pass 46).  (A hand tally of the 3D formulas, 1164, counted multiply-add
-#   pairs the compiler fuses.)
-FP64_OPS_PER_CELL_STEP = {"2d": 94, "3d": 992}
+# division being the Newton-Raphson division with remainder correction, 5):
+#   2D (n_iters = 2, FCT, G = 1), 80, counted from the formulas: pass 1 6 (two face fluxes, three
+#   flux differences, the update), pseudo-velocities 25 per face (A and B 7 each, V_q 3, the
+#   combination 7, the flux 1), FCT 18 (in/out sums 6, two factors 6 each), limited fluxes 2,
+#   pass 2 4 (the 2D kernels execute 96 per cell-step at 1024^2, their recomputed halo included);
+#   3D (n_iters = 3 + tot + FCT + G), 874, counted by ncu as the DADD + DMUL + DFMA instructions of
+#   one step of the staged FP64 kernels at 128^3 (no recomputed halo): pass 1 38, the bounds 0,
+#   per corrective pass 418 (pseudo-advector with the cross and third-order terms 342, factors 32,
+#   limiter 6, donor pass 38).
+FP64_OPS_PER_CELL_STEP = {"2d": 80, "3d": 874}
 
 
 def measure_fma_rates(dev):
@@ -577,8 +576,8 @@ def _events():
 
 def bench_abs(psi_np, gc_np, dtype, dev, stream, flush, steps):
     """The variable-sign option (abs, Sect. 3.1.5) on the rotation workload shifted to cross zero
-    (cone top +1.5 over a background of -1.5), FCT, on the staged kernels (the fused ones
-    decline it): each step timed between CUDA events after an L2 flush, and 10 steps against
+    (cone top +1.5 over a background of -1.5), FCT (FP32: a variant of the fused march; FP64: the
+    staged kernels): each step timed between CUDA events after an L2 flush, and 10 steps against
     the same option in FP64 on the GPU (whose parity with the oracle the tests check)."""
     import numpy as np
     import torch
@@ -605,7 +604,8 @@ def bench_abs(psi_np, gc_np, dtype, dev, stream, flush, steps):
         torch.cuda.synchronize(dev)
         secs = sum(e0.elapsed_time(e1) for e0, e1 in evs) / 1e3
         res = {"value": round(n * n * steps / secs / 1e9, 3), "unit": UNIT, "steps": steps,
-               "workload": f"2d_rotation_{n}x{n}_variable_sign_abs_fct", "path": "staged kernels"}
+               "workload": f"2d_rotation_{n}x{n}_variable_sign_abs_fct",
+               "path": "fused march" if dtype == torch.float32 else "staged kernels"}
         p0 = torch.tensor(psi_v, dtype=dtype, device=dev)
         q = torch.empty_like(p0)
         m.advance(p0, q, gc, n_steps=10)
@@ -623,8 +623,9 @@ def bench_abs(psi_np, gc_np, dtype, dev, stream, flush, steps):
 def bench_dfl(n, dtype, dev, stream, flush, steps):
     """The divergent-flow option (dfl, Sect. 3.1.3) on an n^2 field in the steady separable
     divergent flow u = 1 + 0.5 sin(2 pi x), v = 0.7 (1 + 0.4 cos(2 pi y)) at max |C| 0.25 (the
-    flow of its convergence pin), two passes, on the staged kernels: each step timed between
-    CUDA events after an L2 flush, and 10 steps against FP64 on the GPU."""
+    flow of its convergence pin), two passes (FP32: a variant of the fused march; FP64: the
+    shared-memory tile kernel): each step timed between CUDA events after an L2 flush, and 10
+    steps against FP64 on the GPU."""
     import numpy as np
     import torch
 
@@ -637,7 +638,8 @@ def bench_dfl(n, dtype, dev, stream, flush, steps):
     c = 0.25 / max(u.max(), v.max())
     gc_np = [np.broadcast_to((c * v)[:, None], (n, n)).copy(), np.broadcast_to((c * u)[None, :], (n, n)).copy()]
     opts = capi.DFL
-    res = {"workload": f"2d_divergent_separable_{n}x{n}_dfl_n_iters2", "path": "staged kernels"}
+    res = {"workload": f"2d_divergent_separable_{n}x{n}_dfl_n_iters2",
+           "path": "fused march" if dtype == torch.float32 else "shared-memory tile kernel"}
     outs = {}
     for dt in (dtype, torch.float64):
         with Mpdata((n, n), dtype=dt, n_iters=2, opts=opts, device=dev) as m:
@@ -688,7 +690,8 @@ def bench_config1(dev):
     return {"workload": "1d_box_gaussian_n500_c0.5_n_iters2_f64", "steps": 1000, "time_ms": round(secs * 1e3, 3),
             "value": round(500 * 1000 / secs / 1e9, 4), "unit": UNIT,
             "one_transit_rms_err_vs_initial": float(np.sqrt(np.mean((out - psi) ** 2))),
-            "path": "one launch of one block for all steps (field and intermediates in shared memory; FP64 rate of one SM)"}
+            "path": "one launch of one thread-block cluster for all steps (field in registers, halos through distributed "
+                    "shared memory)"}
 
 
 def bench_config3(dev, n=256, steps=20, oracle_steps=1):
