@@ -158,6 +158,14 @@ using dev::grid_wait;
         const auto i = nb.i;
 #define CELL_END }
 
+// Asks for the cells' lines of an array in L2.  A rollout's tapes exceed the L2, so the first kernel of
+// a reverse sweep finds its inputs in HBM; requested before grid_wait() they arrive while the last
+// kernel of the sweep before ends (a prefetch returns no value, so it may run before the array is written).
+template <typename T>
+__device__ __forceinline__ void prefetch_l2(const T* p) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
+
 // Reverse of the donor-cell pass k, psi_k = psi_{k-1} + sum_d (F_{i-e_d} - F_i)/G_i with
 // F = flux(psi_{k-1}, V^k): pb_prev += dL/dpsi_{k-1}, vhb[d] += dL/dV^k.  FINAL (the first
 // pass, reversed last): the step's outputs are written here instead, psi_out = pb_prev +
@@ -169,6 +177,7 @@ __global__ void ka_donor_flux(Grid g, const T* __restrict__ pb, const T* __restr
                               const T* __restrict__ G, bool unit, T* pb_prev, W3<T> vhb, T* __restrict__ psi_out,
                               W3<T> gc_out, T* zb, int nz, long long zn) {
   grid_wait();
+  if (FINAL) grid_release();  // the next sweep's first kernel starts its prefetches
   CELL_INDEX
   const T gi = G ? adiv(pb[i], G[i]) : pb[i];
   T acc = pb[i];
@@ -477,6 +486,17 @@ __global__ void ka_fct_a(Grid g, const T* __restrict__ pb, const T* __restrict__
                          const T* __restrict__ G, bool unit, const T* __restrict__ bu, const T* __restrict__ bd,
                          const T* __restrict__ mx, const T* __restrict__ mn, bool first, T* __restrict__ pb_prev,
                          W3<T> vb, T* __restrict__ mxb, T* __restrict__ mnb, W3<T> fb) {
+  if (threadIdx.x % (128 / sizeof(T)) == 0) {  // one request per 128-byte line
+    CELL_INDEX
+    prefetch_l2(psi + i);
+#pragma unroll
+    for (int d = 0; d < ND; ++d) prefetch_l2(Vu.p[d] + i);
+    prefetch_l2(bu + i);
+    prefetch_l2(bd + i);
+    prefetch_l2(mx + i);
+    prefetch_l2(mn + i);
+    CELL_END
+  }
   grid_wait();
   grid_release();
   CELL_INDEX
