@@ -173,14 +173,14 @@ __device__ __forceinline__ void prefetch_l2(const T* p) {
 // then the cell's element of each of the nz arrays at zb (stride zn; they include pb_prev
 // and vhb) is cleared for the next reverse step.
 template <typename T, int ND, bool FINAL>
-__global__ void ka_donor_flux(Grid g, const T* __restrict__ pb, const T* __restrict__ psi, P3<T> V,
-                              const T* __restrict__ G, bool unit, T* pb_prev, W3<T> vhb, T* __restrict__ psi_out,
-                              W3<T> gc_out, T* zb, int nz, long long zn) {
+__global__ void ka_donor_flux(Grid g, const T* pb, const T* psi, P3<T> V, const T* G, bool unit, T* pb_prev, W3<T> vhb,
+                              T* psi_out, W3<T> gc_out, T* zb, int nz, long long zn) {
   grid_wait();
   if (FINAL) grid_release();  // the next sweep's first kernel starts its prefetches
   CELL_INDEX
   const T gi = G ? adiv(pb[i], G[i]) : pb[i];
   T acc = pb[i];
+  T w[ND];  // dL/dV on the cell's faces, stored after the last load
 #pragma unroll
   for (int d = 0; d < ND; ++d) {
     const auto ip = nb.at(d, +1), im = nb.at(d, -1);
@@ -194,17 +194,23 @@ __global__ void ka_donor_flux(Grid g, const T* __restrict__ pb, const T* __restr
       acc += fp * posp(v) + fm * negp(vm);
       dv = dpos(v) * psi[i] + dneg(v) * psi[ip];
     }
+    w[d] = fp * dv;
+    if (FINAL && gc_out.p[d]) w[d] = gc_out.p[d][i] + (vhb.p[d][i] + w[d]);
+  }
+  const T before = pb_prev[i];
+#pragma unroll
+  for (int d = 0; d < ND; ++d) {
     if (!FINAL) {
-      vhb.p[d][i] += fp * dv;
+      vhb.p[d][i] += w[d];
     } else if (gc_out.p[d]) {
-      gc_out.p[d][i] += vhb.p[d][i] + fp * dv;
+      gc_out.p[d][i] = w[d];
     }
   }
   if (FINAL) {
-    psi_out[i] = pb_prev[i] + acc;
+    psi_out[i] = before + acc;
     for (int a = 0; a < nz; ++a) zb[a * zn + i] = T(0);
   } else {
-    pb_prev[i] += acc;
+    pb_prev[i] = before + acc;
   }
   CELL_END
 }
@@ -482,10 +488,9 @@ __device__ __forceinline__ T limit_choice(const T F, const T v, const T* __restr
 // bounds adjoints (set on the first pass reversed, accumulated on later ones), and scatters
 // the adjoints of the unlimited fluxes into fb.  Branches follow the forward's choices.
 template <typename T, int ND>
-__global__ void ka_fct_a(Grid g, const T* __restrict__ pb, const T* __restrict__ psi, P3<T> Vu, P3<T> vhs,
-                         const T* __restrict__ G, bool unit, const T* __restrict__ bu, const T* __restrict__ bd,
-                         const T* __restrict__ mx, const T* __restrict__ mn, bool first, T* __restrict__ pb_prev,
-                         W3<T> vb, T* __restrict__ mxb, T* __restrict__ mnb, W3<T> fb) {
+__global__ void ka_fct_a(Grid g, const T* pb, const T* psi, P3<T> Vu, P3<T> vhs, const T* G, bool unit, const T* bu,
+                         const T* bd, const T* mx, const T* mn, bool first, T* pb_prev, W3<T> vb, T* mxb, T* mnb,
+                         W3<T> fb) {
   if (threadIdx.x % (128 / sizeof(T)) == 0) {  // one request per 128-byte line
     CELL_INDEX
     prefetch_l2(psi + i);
@@ -504,7 +509,7 @@ __global__ void ka_fct_a(Grid g, const T* __restrict__ pb, const T* __restrict__
   const T gi = G ? adiv(pb[i], G[i]) : pb[i];
   T acc = pb[i];
   T gu = T(0), gd = T(0);  // adjoints of beta_up and beta_dn of this cell
-  T Fp[3], Fm[3];
+  T Fp[3], Fm[3], w[ND];
   decltype(nb.i) im[3];
 #pragma unroll
   for (int d = 0; d < ND; ++d) {
@@ -531,7 +536,7 @@ __global__ void ka_fct_a(Grid g, const T* __restrict__ pb, const T* __restrict__
     }
     T gq = fp * dv, gqm = fm * dvm;  // dL/dV^ on the two faces
     if (vhs.p[d]) { gq += vhs.p[d][i]; gqm += vhs.p[d][im[d]]; }
-    vb.p[d][i] = gq * m;
+    w[d] = gq * m;  // stored after the last load
     if (sel == 1) (right ? gd : gu) += gq * v;
     if (sel_m == 2) (right_m ? gu : gd) += gqm * vm;
   }
@@ -542,21 +547,24 @@ __global__ void ka_fct_a(Grid g, const T* __restrict__ pb, const T* __restrict__
     ou = ou + (posp(Fp[d]) - negp(Fm[d]));
   }
   const T Gi = G ? G[i] : T(1);
+  const T hi = mx[i], lo = mn[i];
   T gin = T(0), gout = T(0), pacc = T(0), dmx = T(0), dmn = T(0);
   if (gtz(in) && nez(gu)) {
-    const T beta = adiv(Gi * posp(mx[i] - p), in);
-    const T t = adiv(gu * Gi * dpos(mx[i] - p), in);
+    const T beta = adiv(Gi * posp(hi - p), in);
+    const T t = adiv(gu * Gi * dpos(hi - p), in);
     dmx = t;
     pacc -= t;
     gin = adiv(-gu * beta, in);
   }
   if (gtz(ou) && nez(gd)) {
-    const T beta = adiv(Gi * posp(p - mn[i]), ou);
-    const T t = adiv(gd * Gi * dpos(p - mn[i]), ou);
+    const T beta = adiv(Gi * posp(p - lo), ou);
+    const T t = adiv(gd * Gi * dpos(p - lo), ou);
     pacc += t;
     dmn = -t;
     gout = adiv(-gd * beta, ou);
   }
+#pragma unroll
+  for (int d = 0; d < ND; ++d) vb.p[d][i] = w[d];
   if (nez(gin) || nez(gout)) {
 #pragma unroll
     for (int d = 0; d < ND; ++d) {
@@ -604,13 +612,14 @@ __device__ __forceinline__ void bounds_rev(const Nbr<ND>& nb, const decltype(Nbr
 // advector that produced V (Eq. 6, scattered into pb and vhb).  On the last pass reversed
 // (mxb not null) also the bounds over psi^n = p0 and psi^(1) = psi.
 template <typename T, int ND, bool EXT>
-__global__ void ka_fct_b(Grid g, P3<T> fb, P3<T> vbl, const T* __restrict__ psi, P3<T> Vu, P3<T> Vin,
-                         const T* __restrict__ G, bool unit, bool tot, bool abs_psi, bool dfl, T* pb, W3<T> vhb,
-                         const T* __restrict__ mxb, const T* __restrict__ mnb, const T* __restrict__ p0, T* pb0) {
+__global__ void ka_fct_b(Grid g, P3<T> fb, P3<T> vbl, const T* psi, P3<T> Vu, P3<T> Vin, const T* G, bool unit, bool tot,
+                         bool abs_psi, bool dfl, T* pb, W3<T> vhb, const T* mxb, const T* mnb, const T* p0, T* pb0) {
   grid_wait();
   grid_release();
   CELL_INDEX
   T acc = T(0);
+  T w[ND];  // dL/dV on the cell's faces, formed before the first scatter
+  const T gmx = mxb ? mxb[i] : T(0), gmn = mxb ? mnb[i] : T(0);
 #pragma unroll
   for (int d = 0; d < ND; ++d) {
     const auto ip = nb.at(d, +1), im = nb.at(d, -1);
@@ -621,14 +630,18 @@ __global__ void ka_fct_b(Grid g, P3<T> fb, P3<T> vbl, const T* __restrict__ psi,
       acc += fp * posp(v) + fm * negp(vm);
       dv = dpos(v) * psi[i] + dneg(v) * psi[ip];
     }
-    const T gout = vbl.p[d][i] + fp * dv;
+    w[d] = vbl.p[d][i] + fp * dv;
+  }
+#pragma unroll
+  for (int d = 0; d < ND; ++d) {
+    const T gout = w[d];
     if (nez(gout)) {
       if constexpr (EXT) antidiff_face_rev_ext<T, ND>(nb, i, d, gout, psi, Vin, G, unit, tot, abs_psi, dfl, pb, vhb);
       else antidiff_face_rev<T, ND>(nb, i, d, gout, psi, Vin, G, unit, pb, vhb);
     }
   }
   if (nez(acc)) atomicAdd(&pb[i], acc);
-  if (mxb) bounds_rev<T, ND>(nb, i, mxb[i], mnb[i], p0, psi, pb0, pb);
+  if (mxb) bounds_rev<T, ND>(nb, i, gmx, gmn, p0, psi, pb0, pb);
   CELL_END
 }
 

@@ -5,6 +5,14 @@
 // tail.  A kernel calls grid_release() to let its successor's launch begin as soon as every block
 // of its own grid has started.  grid_wait() waits for the whole predecessor, which waited for its
 // own, so everything before a chain is complete too.
+//
+// A kernel that calls grid_wait() is resident while its predecessor still writes, so what a kernel
+// before it in the chain may write (psi, the advectors between the passes, bounds, factors,
+// psi_bar) is read by ordinary loads: no __ldg, and no __restrict__ on the kernel's parameter,
+// with which the compiler may take the array as constant for the whole kernel and read it through
+// the read-only path or before the wait.  Neither is put on what the kernel writes itself.  Both
+// stay for G, R and b, which no kernel of a forward call writes; the reverse sweep's kernels, whose
+// first is a dependent of whatever the caller put on the stream before, have them nowhere.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -81,15 +81,16 @@ struct Plan {
 };
 
 // The lane's NC cells of a row in global memory: one vector (VEC, from column xc[0]), or cell by
-// cell at the wrapped columns xc
+// cell at the wrapped columns xc.  Ordinary loads: a kernel of the same chain may have written the
+// row (launch.cuh)
 template <int NC, bool VEC>
 __device__ __forceinline__ void load_cells(const float* row, const int (&xc)[NC], float (&r)[NC]) {
   if constexpr (VEC && NC == 4) {
-    const float4 v = __ldg(reinterpret_cast<const float4*>(row + xc[0]));
+    const float4 v = *reinterpret_cast<const float4*>(row + xc[0]);
     r[0] = v.x; r[1] = v.y; r[2] = v.z; r[3] = v.w;
   } else {
 #pragma unroll
-    for (int c = 0; c < NC; ++c) r[c] = __ldg(row + xc[c]);
+    for (int c = 0; c < NC; ++c) r[c] = row[xc[c]];
   }
 }
 // The lane's NC cells to a row of nx cells from column xl on (q: the row's element xl)
@@ -207,7 +208,7 @@ constexpr size_t antidiff3v_smem() {
 // NC cells per lane; MINB resident blocks per SM requested from the register allocator; the
 // options are compile-time so that the cells' and faces' arithmetic has no branch between it
 template <int NC, int MINB, bool VEC, int ZC, bool ABS, bool IGA, bool TOT, bool NUG>
-__global__ void __launch_bounds__(kThreads, MINB) k_antidiff3v(Grid g, int zc_any, const float* __restrict__ psi, V3 Vin,
+__global__ void __launch_bounds__(kThreads, MINB) k_antidiff3v(Grid g, int zc_any, const float* psi, V3 Vin,
                                                          float vscale, const float* __restrict__ G, O3 Vout) {
   constexpr int W = row_w<NC>();
   constexpr int nP = kPsiRows * W, nV = kVRows * W;
@@ -429,9 +430,8 @@ __device__ __forceinline__ float donor1(float p, const float (&np)[3], const flo
 }
 
 template <int NC, bool VEC, int ZC, bool KAHAN, bool NUG>
-__global__ void __launch_bounds__(kCThreads, 2) k_p1b3v(Grid g, int zc_any, const float* __restrict__ psi, V3 V, float vscale,
-                                                     const float* __restrict__ G, float* __restrict__ p1,
-                                                     float* __restrict__ mx, float* __restrict__ mn) {
+__global__ void __launch_bounds__(kCThreads, 2) k_p1b3v(Grid g, int zc_any, const float* psi, V3 V, float vscale,
+                                                     const float* __restrict__ G, float* p1, float* mx, float* mn) {
   constexpr int W = row_w<NC>();
   constexpr int nP = kBPsiRows * W, nX = kBVxRows * W, nY = kBVyRows * W, nZ = kBVzRows * W, n1 = kB1Rows * W;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -668,10 +668,9 @@ __device__ __forceinline__ float limited(float L, float R, float V, float buL, f
 }
 
 template <int NC, bool VEC, int ZC, bool NUG, bool UNIT, bool LIM>
-__global__ void __launch_bounds__(kCThreads, 2) k_corr3v(Grid g, int zc_any, const float* __restrict__ psi, V3 Vu,
-                                                         const float* __restrict__ G, const float* __restrict__ mxg,
-                                                         const float* __restrict__ mng, O3 lim,
-                                                         float* __restrict__ out) {
+__global__ void __launch_bounds__(kCThreads, 2) k_corr3v(Grid g, int zc_any, const float* psi, V3 Vu,
+                                                         const float* __restrict__ G, const float* mxg,
+                                                         const float* mng, O3 lim, float* out) {
   constexpr int W = row_w<NC>();
   constexpr int nP = kKPsiRows * W, nV = kKVRows * W, nB = kKBRows * W;
   extern __shared__ __align__(16) unsigned char smem_raw[];

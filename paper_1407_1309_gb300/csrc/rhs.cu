@@ -16,8 +16,8 @@ namespace mpd {
 namespace {
 
 template <typename T>
-__global__ void k_trapez_pre(const TrapezMat m, long long n, T half_dt, const T* __restrict__ psi,
-                             const T* __restrict__ b, T* __restrict__ out) {
+__global__ void k_trapez_pre(const TrapezMat m, long long n, T half_dt, const T* psi, const T* __restrict__ b,
+                             T* out) {
   dev::grid_wait();
   for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
        i += static_cast<long long>(gridDim.x) * blockDim.x) {
@@ -38,8 +38,7 @@ __global__ void k_trapez_pre(const TrapezMat m, long long n, T half_dt, const T*
 }
 
 template <typename T>
-__global__ void k_trapez_post(const TrapezMat m, long long n, T half_dt, const T* __restrict__ b,
-                              T* __restrict__ psi) {
+__global__ void k_trapez_post(const TrapezMat m, long long n, T half_dt, const T* __restrict__ b, T* psi) {
   dev::grid_wait();
   for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
        i += static_cast<long long>(gridDim.x) * blockDim.x) {

@@ -153,8 +153,7 @@ __device__ __forceinline__ T flux(T L, T R, T V, bool unit) {
 }
 
 template <typename T>
-__global__ void k_pre(long long N, const T* __restrict__ psi, const T* __restrict__ r, T dt,
-                      T* __restrict__ out) {
+__global__ void k_pre(long long N, const T* psi, const T* __restrict__ r, T dt, T* out) {
   dev::grid_wait();
   const long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
   if (i < N) out[i] = psi[i] + dt * r[i];
@@ -163,9 +162,8 @@ __global__ void k_pre(long long N, const T* __restrict__ psi, const T* __restric
 // Donor-cell pass (Eqs. 4-5): psi_i - F_{i+1/2}/G_i + F_{i-1/2}/G_i, dimension 0 first,
 // optionally with compensated (Kahan) summation; euler_a source added when post.
 template <typename T, int ND>
-__global__ void k_donor(Grid g, const T* __restrict__ psi, In3<T> V, T vscale, bool unit,
-                        const T* __restrict__ G, bool kahan, const T* __restrict__ R, T dt,
-                        bool post, T* __restrict__ out) {
+__global__ void k_donor(Grid g, const T* psi, In3<T> V, T vscale, bool unit, const T* __restrict__ G, bool kahan,
+                        const T* __restrict__ R, T dt, bool post, T* out) {
   dev::grid_wait();
   FOR_CELLS(g) {
   const Nbr<ND> nb(g, Coord{{c0_, c1_, c2_}});
@@ -203,8 +201,7 @@ __global__ void k_donor(Grid g, const T* __restrict__ psi, In3<T> V, T vscale, b
 
 // FCT bounds (Sect. 3.1.4): extrema of psi0 and psi1 over the cell and its face neighbours.
 template <typename T, int ND>
-__global__ void k_bounds(Grid g, const T* __restrict__ p0, const T* __restrict__ p1,
-                         T* __restrict__ mx, T* __restrict__ mn) {
+__global__ void k_bounds(Grid g, const T* p0, const T* p1, T* mx, T* mn) {
   dev::grid_wait();
   FOR_CELLS(g) {
   const Nbr<ND> nb(g, Coord{{c0_, c1_, c2_}});
@@ -237,8 +234,8 @@ __global__ void k_bounds(Grid g, const T* __restrict__ p0, const T* __restrict__
 // values it uses (over their count under infinite gauge; of their magnitudes with abs_psi,
 // Sect. 3.1.5).
 template <typename T, int ND>
-__global__ void k_antidiff(Grid g, const T* __restrict__ psi, In3<T> Vin, T vscale,
-                           const T* __restrict__ G, bool iga, bool tot, bool abs_psi, bool dfl, Out3<T> Vout) {
+__global__ void k_antidiff(Grid g, const T* psi, In3<T> Vin, T vscale, const T* __restrict__ G, bool iga, bool tot, bool abs_psi,
+                           bool dfl, Out3<T> Vout) {
   dev::grid_wait();
   // variable-sign option (Sect. 3.1.5): psi enters every psi-fraction as |psi|
   auto ps = [&](long long j) { const T v = psi[j]; return abs_psi ? absv(v) : v; };
@@ -246,6 +243,7 @@ __global__ void k_antidiff(Grid g, const T* __restrict__ psi, In3<T> Vin, T vsca
   const Nbr<ND> nb(g, Coord{{c0_, c1_, c2_}});
   const long long i = nb.i;
   const T p0 = ps(i);
+  T res[ND];
 #pragma unroll
   for (int d = 0; d < ND; ++d) {
     const long long ip = nb.at(d, +1);
@@ -319,8 +317,11 @@ __global__ void k_antidiff(Grid g, const T* __restrict__ psi, In3<T> Vin, T vsca
       }
       out = out - T(0.25) * V * div * rGb;
     }
-    Vout.p[d][i] = out;
+    res[d] = out;
   }
+  // stored after all faces, so that no store separates the loads (psi may alias what is stored)
+#pragma unroll
+  for (int d = 0; d < ND; ++d) Vout.p[d][i] = res[d];
   }
 }
 
@@ -376,7 +377,7 @@ __device__ __forceinline__ int rot(int s, int j, int n) {
 }
 
 template <typename T, bool ABS>
-__global__ void __launch_bounds__(kAx * kAy) k_antidiff3(Grid g, const T* __restrict__ psi, In3<T> Vin,
+__global__ void __launch_bounds__(kAx * kAy) k_antidiff3(Grid g, const T* psi, In3<T> Vin,
                                                          T vscale, const T* __restrict__ G, bool iga, bool tot,
                                                          Out3<T> Vout) {
   dev::grid_wait();
@@ -588,9 +589,8 @@ constexpr size_t p1b3_smem() {
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kAx * kAy) k_p1b3(Grid g, const T* __restrict__ psi, In3<T> V, T vscale,
-                                                    const T* __restrict__ G, bool kahan, T* __restrict__ p1,
-                                                    T* __restrict__ mx, T* __restrict__ mn) {
+__global__ void __launch_bounds__(kAx * kAy) k_p1b3(Grid g, const T* psi, In3<T> V, T vscale,
+                                                    const T* __restrict__ G, bool kahan, T* p1, T* mx, T* mn) {
   dev::grid_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int nB = kBw * kBh, nX = kXw * kXh, nH = kHw * kHh;
@@ -759,11 +759,9 @@ constexpr size_t corr3_smem() {
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kAx * kAy) k_corr3(Grid g, const T* __restrict__ psi, In3<T> Vu,
-                                                     const T* __restrict__ G, bool unit, bool kahan,
-                                                     const T* __restrict__ mxg, const T* __restrict__ mng,
-                                                     const T* __restrict__ R, T dt, bool post, Out3<T> lim,
-                                                     T* __restrict__ out) {
+__global__ void __launch_bounds__(kAx * kAy) k_corr3(Grid g, const T* psi, In3<T> Vu, const T* __restrict__ G,
+                                                     bool unit, bool kahan, const T* mxg, const T* mng,
+                                                     const T* __restrict__ R, T dt, bool post, Out3<T> lim, T* out) {
   dev::grid_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* const sm = reinterpret_cast<T*>(smem_raw);
@@ -1001,9 +999,8 @@ __global__ void __launch_bounds__(kAx * kAy) k_corr3(Grid g, const T* __restrict
 // FCT limiting factors (Sect. 3.1.4): in/out sums of the unlimited fluxes and
 // beta_up = G [psi_max - psi]+ / in, beta_dn = G [psi - psi_min]+ / out (1 when the sum is 0).
 template <typename T, int ND>
-__global__ void k_beta(Grid g, const T* __restrict__ psi, In3<T> V, const T* __restrict__ G, bool unit,
-                       const T* __restrict__ mx, const T* __restrict__ mn, T* __restrict__ bu,
-                       T* __restrict__ bd) {
+__global__ void k_beta(Grid g, const T* psi, In3<T> V, const T* __restrict__ G, bool unit, const T* mx, const T* mn,
+                       T* bu, T* bd) {
   dev::grid_wait();
   FOR_CELLS(g) {
   const Nbr<ND> nb(g, Coord{{c0_, c1_, c2_}});
@@ -1020,21 +1017,23 @@ __global__ void k_beta(Grid g, const T* __restrict__ psi, In3<T> V, const T* __r
     out = out + (posp(Fp) - negp(Fm));
   }
   const T Gi = G ? G[i] : T(1);
-  bu[i] = factor_sum(in) ? qdiv(Gi * posp(mx[i] - p), in) : T(1);
-  bd[i] = factor_sum(out) ? qdiv(Gi * posp(p - mn[i]), out) : T(1);
+  const T up = factor_sum(in) ? qdiv(Gi * posp(mx[i] - p), in) : T(1);
+  const T dn = factor_sum(out) ? qdiv(Gi * posp(p - mn[i]), out) : T(1);
+  bu[i] = up;
+  bd[i] = dn;
   }
 }
 
 // Limited advector: V min(1, beta_dn_i, beta_up_{i+e_d}) if the unlimited flux leaves
 // cell i (F > 0, or F = 0 with V > 0), else V min(1, beta_up_i, beta_dn_{i+e_d}).
 template <typename T, int ND>
-__global__ void k_limit(Grid g, const T* __restrict__ psi, In3<T> Vu, bool unit,
-                        const T* __restrict__ bu, const T* __restrict__ bd, Out3<T> Vout) {
+__global__ void k_limit(Grid g, const T* psi, In3<T> Vu, bool unit, const T* bu, const T* bd, Out3<T> Vout) {
   dev::grid_wait();
   FOR_CELLS(g) {
   const Nbr<ND> nb(g, Coord{{c0_, c1_, c2_}});
   const long long i = nb.i;
   const T p = psi[i];
+  T res[ND];
 #pragma unroll
   for (int d = 0; d < ND; ++d) {
     const long long ip = nb.at(d, +1);
@@ -1046,8 +1045,10 @@ __global__ void k_limit(Grid g, const T* __restrict__ psi, In3<T> Vu, bool unit,
     T m = T(1);
     m = mine(a, m);
     m = mine(b, m);
-    Vout.p[d][i] = V * m;
+    res[d] = V * m;
   }
+#pragma unroll
+  for (int d = 0; d < ND; ++d) Vout.p[d][i] = res[d];
   }
 }
 

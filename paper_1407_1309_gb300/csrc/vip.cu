@@ -36,8 +36,8 @@ __device__ __forceinline__ long long nb(const Grid& g, const int (&c)[3], long l
 }
 
 template <typename T>
-__global__ void k_vip_cells(long long n, int nd, const T* __restrict__ state, T* __restrict__ uprev,
-                            T* __restrict__ ext, bool first, T eps) {
+__global__ void k_vip_cells(long long n, int nd, const T* state, T* uprev,
+                            T* ext, bool first, T eps) {
   dev::grid_wait();
   for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
        i += static_cast<long long>(gridDim.x) * blockDim.x) {
@@ -52,7 +52,7 @@ __global__ void k_vip_cells(long long n, int nd, const T* __restrict__ state, T*
 }
 
 template <typename T>
-__global__ void k_vip_faces(Grid g, const T* __restrict__ ext, T* __restrict__ adv, T courant) {
+__global__ void k_vip_faces(Grid g, const T* ext, T* adv, T courant) {
   dev::grid_wait();
   const long long n = g.N;
   for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
@@ -68,7 +68,7 @@ __global__ void k_vip_faces(Grid g, const T* __restrict__ ext, T* __restrict__ a
 }
 
 template <typename T>
-__global__ void k_sw_force(Grid g, T* __restrict__ state, T half_dt, T inv2dx) {
+__global__ void k_sw_force(Grid g, T* state, T half_dt, T inv2dx) {
   dev::grid_wait();
   const long long n = g.N;
   for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
