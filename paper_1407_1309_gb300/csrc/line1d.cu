@@ -81,8 +81,8 @@ __device__ __forceinline__ void remote_store(const double* p, unsigned rank, dou
 template <typename T> __device__ __forceinline__ T up1(T x) { return __shfl_up_sync(kFull, x, 1); }
 template <typename T> __device__ __forceinline__ T down1(T x) { return __shfl_down_sync(kFull, x, 1); }
 
-// a flux sum that takes a limiting factor (0 or a subnormal sum gives the factor 1)
-__device__ __forceinline__ bool positive_sum(float x) { return x >= 1.17549435e-38f; }
+// a flux sum that takes a limiting factor (0, or in FP64 a subnormal sum, gives the factor 1)
+__device__ __forceinline__ bool positive_sum(float x) { return x > 0.0f; }
 __device__ __forceinline__ bool positive_sum(double x) { return gt0(x) && divisible(x); }
 __device__ __forceinline__ bool is_zero(float x) { return x == 0.0f; }
 __device__ __forceinline__ bool is_zero(double x) { return !nonzero(x); }

@@ -144,7 +144,7 @@ __device__ __forceinline__ void put(float* dst, const float (&v)[NC]) {
   else *reinterpret_cast<float2*>(dst) = make_float2(v[0], v[1]);
 }
 
-__device__ __forceinline__ float frac1(float n, float d) { return divisible(d) ? fdiv(n, d) : 0.0f; }
+__device__ __forceinline__ float frac1(float n, float d) { return ratio(n, d); }
 // n1/d and n2/d with one guard and one approximate reciprocal (0 when d == 0)
 __device__ __forceinline__ void frac2v(float n1, float n2, float d, float& r1, float& r2) {
   const float r = rcp(d);

@@ -32,7 +32,7 @@ template <> __device__ __forceinline__ float qdiv<float>(float n, float d) { ret
 template <> __device__ __forceinline__ double qdiv<double>(double n, double d) { return dev::nr_div(n, d); }
 // psi-fraction with the zero-denominator guard (the ratio of Eq. 6 is 0 when its sum is 0)
 // (a divisor below the smallest normal number counts as zero: stencil2d.cuh)
-template <typename T> __device__ __forceinline__ T fracg(T n, T d) { return dev::divisible(d) ? qdiv(n, d) : T(0); }
+template <typename T> __device__ __forceinline__ T fracg(T n, T d) { return dev::ratio(n, d); }
 // FP32: single min/max instructions; FP64: the sign tests, extrema and |x| on the integer pipe
 // (stencil2d.cuh)
 template <> __device__ __forceinline__ float posp<float>(float x) { return dev::posp(x); }
@@ -48,9 +48,9 @@ __device__ __forceinline__ bool goes_right(float F, float V) { return F > 0.0f |
 __device__ __forceinline__ bool goes_right(double F, double V) {
   return dev::gt0(F) || (!dev::nonzero(F) && dev::gt0(V));
 }
-// a flux sum that takes a limiting factor (0 or a subnormal sum gives the factor 1: the FP64
-// division has no reciprocal of a subnormal, and such a sum cannot move the cell's value)
-__device__ __forceinline__ bool factor_sum(float x) { return x >= 1.17549435e-38f; }
+// a flux sum that takes a limiting factor (0, or in FP64 a subnormal sum, gives the factor 1: the
+// FP64 division has no reciprocal of a subnormal, and such a sum cannot move the cell's value)
+__device__ __forceinline__ bool factor_sum(float x) { return x > 0.0f; }
 __device__ __forceinline__ bool factor_sum(double x) { return dev::gt0(x) && dev::divisible(x); }
 
 template <typename T> struct In3 { const T* p[3]; };

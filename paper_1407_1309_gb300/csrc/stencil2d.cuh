@@ -17,17 +17,22 @@ __device__ __forceinline__ int wrapi(int c, int n) {
 }
 
 template <typename T> __device__ __forceinline__ T fdiv(T a, T b);
-// FP32 n / d: the approximate reciprocal, subnormals flushed, and a multiply (2 ulp).  The
-// flushing form is one instruction; the non-flushing one (and __fdividef) wraps it in a compare
-// and two scalings for subnormal divisors, which no divisor here needs: the psi-fractions guard
-// them (divisible()), and a flux sum below the smallest normal number gives inf or NaN, which
-// min(1, x) maps to the factor 1.
+// FP32 n / d (2 ulp), also for a d below the smallest normal number: the limiter divides by flux
+// sums, which become that small in the tail of a field.
+template <> __device__ __forceinline__ float fdiv<float>(float a, float b) { return __fdividef(a, b); }
+// Approximate FP32 reciprocals.  rcp() takes and gives subnormal numbers; rcp_normal() flushes them to
+// zero and is for a divisor known to be normal whose quotient is 0 above 2^126, as __fdividef's is
+// (the psi-fractions: divisible()).
 __device__ __forceinline__ float rcp(float d) {
+  float r;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(d));
+  return r;
+}
+__device__ __forceinline__ float rcp_normal(float d) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
   return r;
 }
-template <> __device__ __forceinline__ float fdiv<float>(float a, float b) { return a * rcp(b); }
 // FP64 n / d for the arithmetic-bound FP64 kernels, five FP64 operations: one Newton-Raphson
 // iteration r <- r + r (1 - d r) (quadratic convergence) from the PTX approximate FP64 reciprocal
 // (rcp.approx.ftz.f64, full exponent range), and Markstein's remainder correction
@@ -93,6 +98,9 @@ __device__ __forceinline__ bool divisible(double d) { return ((__double_as_longl
 
 // psi-fraction of Eq. 6 with the zero-denominator guard
 template <typename T> __device__ __forceinline__ T ratio(T n, T d) { return divisible(d) ? fdiv(n, d) : T(0); }
+template <> __device__ __forceinline__ float ratio<float>(float n, float d) {
+  return divisible(d) ? n * rcp_normal(d) : 0.0f;
+}
 
 // x > 0 (the upwind choice of a flux, the limiter's direction)
 __device__ __forceinline__ bool gt0(float x) { return x > 0.0f; }

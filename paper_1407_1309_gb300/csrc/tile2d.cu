@@ -85,7 +85,7 @@ __device__ __forceinline__ Off offs(bool edge, int x, int n, int s) {
 
 // n1/d and n2/d (0 for d = 0) with one guard
 __device__ __forceinline__ void ratio2(float n1, float n2, float d, float& r1, float& r2) {
-  const float r = rcp(d);
+  const float r = rcp_normal(d);
   r1 = divisible(d) ? n1 * r : 0.0f;
   r2 = divisible(d) ? n2 * r : 0.0f;
 }
@@ -93,7 +93,7 @@ __device__ __forceinline__ void ratio2(double n1, double n2, double d, double& r
   r1 = ratio(n1, d);
   r2 = ratio(n2, d);
 }
-__device__ __forceinline__ bool sum_counts(float x) { return x >= 1.17549435e-38f; }
+__device__ __forceinline__ bool sum_counts(float x) { return x > 0.0f; }
 __device__ __forceinline__ bool sum_counts(double x) { return gt0(x) && divisible(x); }
 __device__ __forceinline__ bool zero(float x) { return x == 0.0f; }
 __device__ __forceinline__ bool zero(double x) { return !nonzero(x); }
