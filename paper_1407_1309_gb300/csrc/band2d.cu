@@ -178,10 +178,7 @@ __global__ void __launch_bounds__(W * 32, 2) k_band2d(const BandParams<T> p) {
 
   // the first chunks: what no earlier step of the call writes, then, once the step before this one
   // is complete, psi (the copies of the first part join the first chunk's group)
-  // FP64 blocks are bound by their SM's FP64 pipe: released early only where two steps' blocks fit the
-  // GPU with one per SM (190 x 175, 96 blocks: 27.9 us per step released early, 19.3 not; 25.0 with ordinary
-  // launches)
-  if (gridDim.x <= (sizeof(T) == 4 ? kChainBlocks : kChainBlocks / 2)) grid_release();
+  grid_release_small<T>(gridDim.x);
   if (!p.early) grid_wait();
 #pragma unroll
   for (int j = 0; j < kDepth; ++j) load_row(j * W + w, kRest);

@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_fused2d_batched(const BatchPara
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   T* ring = reinterpret_cast<T*>(smem_raw) + static_cast<size_t>(wib) * kSlots * kArr * cols<NC>();
-  if (gridDim.x <= kChainBlocks) grid_release();
+  grid_release_small<T>(gridDim.x);
   grid_wait();  // the step before this one, when launched as its dependent
   const int total = gridDim.x * kWarps;
   for (int item = blockIdx.x * kWarps + wib; item < b.n_items; item += total) {

@@ -32,7 +32,17 @@ __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.la
 // 2 us step in which an ordinary launch waits for its predecessor.  Measured, ordinary -> chained
 // launches: 59 x 61 (8 blocks) 6.1 -> 3.5 us per step, 512^2 8.5 -> 5.4, plain 1024^2 12.6 -> 10.5,
 // compensated 15.0 -> 13.3, |psi| on 1021 x 1000 12.3 -> 10.8.
+//
+// FP64 blocks are bound by their SM's FP64 pipe, so that two on one SM while another has none cost
+// twice the time: they are never released early.  Measured, released early up to 152 blocks -> not:
+// band march 190 x 175 (96 blocks) 29.7 -> 19.4 us per step, 96^2 14.1 -> 9.8; tile kernel 256^2 with
+// three passes and the limiter (128 blocks) 82 -> 61; ensemble of 16 fields of 128^2 in tiles of 12 rows
+// (132 blocks) 137 -> 99; and with few blocks no difference (59 x 61 9.8, 9.8).
 constexpr unsigned kChainBlocks = 152;
+template <typename T>
+__device__ __forceinline__ void grid_release_small(unsigned blocks) {
+  if (sizeof(T) == 4 && blocks <= kChainBlocks) dev::grid_release();
+}
 
 // kern<<<grid, block, smem, st>>>(args...), as a dependent of the kernel before it where `chained`
 template <typename... KArgs, typename... Args>

@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_fused2d(const F2Params<T> p) {
   constexpr int kArr = arrs<COMP>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  if (gridDim.x <= kChainBlocks) grid_release();
+  grid_release_small<T>(gridDim.x);
   grid_wait();  // the step before this one, when launched as its dependent
   const long long wid = static_cast<long long>(blockIdx.x) * kWarps + wib;
   if (wid >= static_cast<long long>(p.strips) * p.rowtiles) return;  // whole warp

@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(kThreadsT, 2) k_tile2d(const TileParams<T> p) 
   auto inside = [&](int r, int c) {
     return !(e0 && (x0 + r < 0 || x0 + r >= p.n0)) && !(e1 && (y0 + c < 0 || y0 + c >= p.n1));
   };
-  if (gridDim.x * gridDim.y * gridDim.z <= kChainBlocks) grid_release();
+  grid_release_small<T>(gridDim.x * gridDim.y * gridDim.z);
   grid_wait();
   over(0, kRows + 2 * H, 0, L, [&](int r, int c) {
     if (!inside(r, c)) return;

@@ -1,0 +1,49 @@
+"""Rules of the dispatch that only show in time, measured on the device (median of CUDA-event
+times, the sides in turn).  The bounds leave room for noise: each faulty rule was at least 20 %
+slower than the other side."""
+import pytest
+import torch
+
+from paper_1407_1309_gb300 import capi
+from paper_1407_1309_gb300.solver import Mpdata
+
+pytestmark = pytest.mark.gpu
+DEV = torch.device("cuda")
+
+
+def problem(shapes, dtype, n_iters, opts, knobs=None):
+    """A call of 4 steps of random fields, ready to be timed."""
+    one = not isinstance(shapes, list)
+    total = sum(s[0] * s[1] for s in ([shapes] if one else shapes))
+    gen = torch.Generator(device=DEV).manual_seed(1)
+    psi = 2 + torch.rand(total, generator=gen, device=DEV, dtype=dtype)
+    gc = [0.4 * (torch.rand(total, generator=gen, device=DEV, dtype=dtype) - 0.5) for _ in range(2)]
+    if one:
+        psi, gc = psi.reshape(shapes), [v.reshape(shapes) for v in gc]
+    out = torch.empty_like(psi)
+    m = Mpdata(shapes, dtype=dtype, n_iters=n_iters, opts=opts)
+    for k, v in (knobs or {}).items():
+        m.tune(k, v)
+    return lambda: m.advance(psi, out, gc, n_steps=4)
+
+
+def times(*calls):
+    """Median microseconds of each call, timed in turn."""
+    got = [[] for _ in calls]
+    for rep in range(24):
+        for call, ts in zip(calls, got):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            call()
+            b.record()
+            b.synchronize()
+            if rep >= 4:
+                ts.append(a.elapsed_time(b) * 1e3)
+    return [sorted(ts)[len(ts) // 2] for ts in got]
+
+
+def test_fp64_tiles_of_one_per_sm_take_the_time_of_one():
+    """128 blocks, fewer than SMs, take no longer than 8 (the next step's blocks do not crowd them)."""
+    k = {capi.TUNE_KERNEL: 1}
+    few, many = times(problem((64, 64), torch.float64, 3, capi.FCT, k), problem((256, 256), torch.float64, 3, capi.FCT, k))
+    assert many <= 1.15 * few
