@@ -54,6 +54,47 @@ void batched_free(mpdata_s* h) {
   }
 }
 
+namespace {
+
+// The handle's table for lanes of nc columns and tiles of ty rows, in place of the one it has.
+int build_table(mpdata_s* h, int nc, int ty) {
+  batched_free(h);
+  const int nf = handle_fields(h);
+  const Grid* grids = handle_grids(h);
+  const long long* offs = handle_offsets(h);
+  const int stride = fused_strip_stride(nc);
+  std::vector<BatchField> fields(nf);
+  std::vector<int> item_field;
+  for (int f = 0; f < nf; ++f) {
+    BatchField& b = fields[f];
+    b.offset = offs[f];
+    b.n0 = grids[f].n[1];
+    b.n1 = grids[f].n[2];
+    b.strips = (b.n1 + stride - 1) / stride;
+    b.item_base = static_cast<int>(item_field.size());
+    b.vec = (b.n1 % nc == 0) && (b.offset % nc == 0);
+    const long long items = static_cast<long long>(b.strips) * ((b.n0 + ty - 1) / ty);
+    if (item_field.size() + items > (1LL << 30)) return MPDATA_EUNSUPPORTED;
+    item_field.insert(item_field.end(), static_cast<size_t>(items), f);
+  }
+  auto* th = new TableHolder;
+  th->nc = nc;
+  th->tab.ty = ty;
+  th->tab.n_items = static_cast<int>(item_field.size());
+  if (cudaMalloc(&th->tab.fields, sizeof(BatchField) * nf) != cudaSuccess ||
+      cudaMalloc(&th->tab.item_field, sizeof(int) * item_field.size()) != cudaSuccess) {
+    cudaFree(th->tab.fields);
+    delete th;
+    return MPDATA_ENOMEM;
+  }
+  cudaMemcpy(th->tab.fields, fields.data(), sizeof(BatchField) * nf, cudaMemcpyHostToDevice);
+  cudaMemcpy(th->tab.item_field, item_field.data(), sizeof(int) * item_field.size(), cudaMemcpyHostToDevice);
+  *handle_batch(h) = th;
+  return MPDATA_OK;
+}
+
+}  // namespace
+
 template <typename T>
 int batched_step(mpdata_s* h, const T* psi_in, T* psi_out, const T* const* gc, const T* g, const T* r, T dt,
                  T gc_scale, bool chained, const Opts& o) {
@@ -77,40 +118,14 @@ int batched_step(mpdata_s* h, const T* psi_in, T* psi_out, const T* const* gc, c
       }
     }
     if (o.tile_rows > 0) ty = o.tile_rows;
-    batched_free(h);
-    const int nf = handle_fields(h);
-    const Grid* grids = handle_grids(h);
-    const long long* offs = handle_offsets(h);
-    const int stride = fused_strip_stride(nc);
-    std::vector<BatchField> fields(nf);
-    std::vector<int> item_field;
-    for (int f = 0; f < nf; ++f) {
-      BatchField& b = fields[f];
-      b.offset = offs[f];
-      b.n0 = grids[f].n[1];
-      b.n1 = grids[f].n[2];
-      b.strips = (b.n1 + stride - 1) / stride;
-      b.item_base = static_cast<int>(item_field.size());
-      b.vec = (b.n1 % nc == 0) && (b.offset % nc == 0);
-      const long long items = static_cast<long long>(b.strips) * ((b.n0 + ty - 1) / ty);
-      if (item_field.size() + items > (1LL << 30)) return MPDATA_EUNSUPPORTED;
-      item_field.insert(item_field.end(), static_cast<size_t>(items), f);
+    // a setting that asks for the table there is keeps it: graphs captured from earlier calls read it
+    if (th == nullptr || th->nc != nc || th->tab.ty != ty) {
+      const int rc = build_table(h, nc, ty);
+      if (rc != MPDATA_OK) return rc;
+      th = static_cast<TableHolder*>(*slot);
     }
-    th = new TableHolder;
-    th->nc = nc;
     th->rows = o.tile_rows;
     th->kernel = o.kernel;
-    th->tab.ty = ty;
-    th->tab.n_items = static_cast<int>(item_field.size());
-    if (cudaMalloc(&th->tab.fields, sizeof(BatchField) * nf) != cudaSuccess ||
-        cudaMalloc(&th->tab.item_field, sizeof(int) * item_field.size()) != cudaSuccess) {
-      cudaFree(th->tab.fields);
-      delete th;
-      return MPDATA_ENOMEM;
-    }
-    cudaMemcpy(th->tab.fields, fields.data(), sizeof(BatchField) * nf, cudaMemcpyHostToDevice);
-    cudaMemcpy(th->tab.item_field, item_field.data(), sizeof(int) * item_field.size(), cudaMemcpyHostToDevice);
-    *slot = th;
   }
   return fused_batched_step<T>(th->tab, o, psi_in, psi_out, gc[0], gc[1], g, r, dt, gc_scale, chained, handle_stream(h),
                                th->nc);
