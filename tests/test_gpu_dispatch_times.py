@@ -47,3 +47,11 @@ def test_fp64_tiles_of_one_per_sm_take_the_time_of_one():
     k = {capi.TUNE_KERNEL: 1}
     few, many = times(problem((64, 64), torch.float64, 3, capi.FCT, k), problem((256, 256), torch.float64, 3, capi.FCT, k))
     assert many <= 1.15 * few
+
+
+@pytest.mark.parametrize("shapes", [[(200, 200)] * 64, [(60 + 7 * k % 241, 60 + 53 * k % 241) for k in range(100)]],
+                         ids=["64_of_200", "100_of_60_to_300"])
+def test_fp64_ensembles_take_a_tile_height_near_the_best(shapes):
+    rows = (0, 12, 16, 24, 32, 48)
+    got = times(*[problem(shapes, torch.float64, 2, capi.FCT, {capi.TUNE_TILE_ROWS: r}) for r in rows])
+    assert got[0] <= 1.1 * min(got[1:]), dict(zip(rows, got))
