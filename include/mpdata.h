@@ -153,7 +153,8 @@ int mpdata_sw_reset(mpdata_t h);
 /*
  * Advances psi in place by n_steps >= 1 steps (the paper's advance(), Sect. 3.2.5).
  * 2D steps run fused kernels (one launch per step; more than two passes, the third-order terms and
- * open edges as a shared-memory tile kernel), 1D fields short enough for
+ * open edges as a shared-memory tile kernel where that should be faster than one kernel per
+ * sub-step, MPDATA_TUNE_KERNEL), 1D fields short enough for
  * one thread-block cluster (about 10000 cells with two passes) run the whole call in one launch,
  * and so do such 1D systems with trapezoidal sources; the rest run one kernel per sub-step.
  * gc (host array of ndims device pointers): advector components, constant over
@@ -305,7 +306,10 @@ int mpdata_clear_stop(mpdata_t h);
  *   the warps on a small field; for the FP64 fields, whose lanes already own 2, the warp
  *   march).  Batched handles always use the warp march's persistent kernel, for FP32 with lanes of
  *   2 columns when this knob is 3, and with whichever should be faster when it is 0 and the tile
- *   height automatic (4 otherwise).
+ *   height automatic (4 otherwise).  2D steps that neither march covers (third-order terms, more
+ *   than two passes, open edges, FP64 divergent flow): 0 = the shared-memory tile kernel or one
+ *   kernel per sub-step, whichever should be faster; other values = the tile kernel wherever its
+ *   shared memory fits.
  * MPDATA_TUNE_STEPS_PER_LAUNCH: fusion depth S (temporal blocking): 0 or 1 = one step per
  *   launch; 2..4 = mpdata_advance runs its steps in groups of S per launch (the last group
  *   the remainder), each block loading its tile with a 3S-cell halo into shared memory once and

@@ -1,16 +1,19 @@
 // One step of 2D fields as a shared-memory tile kernel: every option and any number of passes
 // whose reach fits, open edges included.  It takes the cases that the register marches
-// (march2d.cuh, band2d.cu) leave: the third-order terms, more than two passes, open edges,
-// and in FP64 the divergent-flow option.
+// (march2d.cuh, band2d.cu) leave, the third-order terms, more than two passes, open edges
+// and in FP64 the divergent-flow option, where it is the faster one: the staged kernels keep FP64
+// fields below about 200^2 and most steps whose halo costs more than their launches (tile_cost.h).
 //
 // Why a tile: those cases ran as one kernel per sub-step (4 launches per pass), each reading every
 // neighbour again through L1 and L2; the shallow-water step of three 320^2 FP64 fields took 22
 // launches.  A block loads the step's input once with its halo, H = 1 + (n_iters - 1) r cells (r: 1,
 // one more with the limiter, one more with the third-order terms), runs the sub-steps there,
 // separated by block barriers, on regions that shrink towards the tile, and writes the tile.  The
-// price is the recomputed halo (1.2x the arithmetic for a 32 x 16 tile with H = 3).  FP64 is bound by
-// the FP64 pipe, FP32 by shared-memory issue.  Fields of one shape with one advector (the
-// shallow-water system) share a launch, one grid layer each.
+// price is the recomputed halo (1.2x the arithmetic for a 32 x 16 tile with H = 3).  32-row tiles repeat
+// less of it than 16-row tiles, which give a small FP64 field more blocks (576^2, third-order terms and
+// limiter: 200 us in 32 rows, 176 in 16; 544^2 135 and 143).  FP64 is bound by the FP64 pipe, FP32 by
+// shared-memory issue.  Fields of one shape with one advector (the shallow-water system) share a
+// launch, one grid layer each.
 //
 // Measured: a shallow-water step of three 320^2 FP64 fields with open edges, |psi|, limiter and
 // divergent-flow term 218 us staged, 96 here with its source kernels (the FP64 pipe's floor is about
@@ -27,6 +30,7 @@
 #include "kernels.h"
 #include "launch.cuh"
 #include "stencil2d.cuh"
+#include "tile_cost.h"
 
 namespace mpd {
 namespace {
@@ -34,7 +38,7 @@ namespace {
 using namespace dev;
 
 constexpr int kThreadsT = 256;
-constexpr int kCols = 32;  // tile columns; rows: 32, or 16 (FP64 fields with too few tiles of 32)
+constexpr int kCols = kTileCols;  // tile columns; rows: 32, or in FP64 16 (tile_rows)
 
 template <typename T>
 struct TileParams {
@@ -304,18 +308,14 @@ __global__ void __launch_bounds__(kThreadsT, 2) k_tile2d(const TileParams<T> p) 
 }
 
 template <typename T, int kRows, bool FCT, bool IGA, bool NUG>
-int launch_rows(const TileParams<T>& p, int fields, cudaStream_t st) {
-  const size_t arrays = 6 + (FCT ? 2 + (p.K > 2 ? 2 : 0) : 0) + (NUG ? 1 : 0) + (p.dfl ? 1 : 0);
-  const size_t smem = sizeof(T) * arrays * (kRows + 2 * p.H) * (kCols + 2 * p.H);
-  static PerDevice<int> most_of;
-  const int most = most_of.get([](int dev) {
-    int m = 0;
-    cudaDeviceGetAttribute(&m, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    cudaFuncSetAttribute(k_tile2d<T, kRows, FCT, IGA, NUG>, cudaFuncAttributeMaxDynamicSharedMemorySize, m);
-    return m;
+int launch_rows(const TileParams<T>& p, int fields, size_t smem, int most, cudaStream_t st) {
+  static PerDevice<bool> attr;
+  attr.get([&](int) {
+    return cudaFuncSetAttribute(k_tile2d<T, kRows, FCT, IGA, NUG>, cudaFuncAttributeMaxDynamicSharedMemorySize, most) ==
+           cudaSuccess;
   });
   const long long ty = (p.n0 + kRows - 1) / kRows;
-  if (smem > static_cast<size_t>(most) || ty > 65535) return MPDATA_EUNSUPPORTED;
+  if (ty > 65535) return MPDATA_EUNSUPPORTED;
   const dim3 grid(static_cast<unsigned>((p.n1 + kCols - 1) / kCols), static_cast<unsigned>(ty),
                   static_cast<unsigned>(fields));
   launch_chained(p.chained, k_tile2d<T, kRows, FCT, IGA, NUG>, grid, dim3(kThreadsT), smem, st, p);
@@ -323,20 +323,21 @@ int launch_rows(const TileParams<T>& p, int fields, cudaStream_t st) {
 }
 
 template <typename T, bool FCT, bool IGA, bool NUG>
-int launch_tile(const TileParams<T>& p, int fields, cudaStream_t st) {
+int launch_tile(const TileParams<T>& p, int fields, bool always, cudaStream_t st) {
+  static PerDevice<int> most_of;
+  const int most = most_of.get([](int dev) {
+    int m = 0;
+    cudaDeviceGetAttribute(&m, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    return m;
+  });
+  const TileCase c{p.n0, p.n1, fields, p.K, FCT, p.tot, NUG, p.dfl, sizeof(T) == 8};
+  const int rows = tile_rows(c, static_cast<size_t>(most), always);
+  if (rows == 0) return MPDATA_EUNSUPPORTED;
+  const size_t smem = tile_smem(c, rows);
   if constexpr (sizeof(T) == 8) {
-    // 32 rows repeat less of the halo's arithmetic (1.13x instead of 1.2x with H = 3), 16 rows feed
-    // more SMs: the taller tile where it leaves nearly every SM two blocks and its shared memory
-    // fits
-    const long long tall = static_cast<long long>(fields) * ((p.n0 + 31) / 32) * ((p.n1 + kCols - 1) / kCols);
-    if (tall >= 280) {
-      const int rc = launch_rows<T, 32, FCT, IGA, NUG>(p, fields, st);
-      if (rc != MPDATA_EUNSUPPORTED) return rc;
-    }
-    return launch_rows<T, 16, FCT, IGA, NUG>(p, fields, st);
-  } else {
-    return launch_rows<T, 32, FCT, IGA, NUG>(p, fields, st);
+    if (rows == 16) return launch_rows<T, 16, FCT, IGA, NUG>(p, fields, smem, most, st);
   }
+  return launch_rows<T, 32, FCT, IGA, NUG>(p, fields, smem, most, st);
 }
 
 }  // namespace
@@ -358,8 +359,9 @@ int tile2d_step(const Grid& g, const Opts& o, const StepArgs<T>& a, int fields, 
   p.n0 = g.n[1];
   p.n1 = g.n[2];
   p.K = o.n_iters;
-  p.reach = 1 + (o.fct ? 1 : 0) + (o.tot ? 1 : 0);
-  p.H = 1 + (p.K - 1) * p.reach;
+  const TileCase c{p.n0, p.n1, fields, p.K, o.fct, o.tot, o.nug, o.dfl, sizeof(T) == 8};
+  p.reach = tile_reach(c);
+  p.H = tile_halo(c);
   p.dt = a.dt;
   p.scale = a.gc_scale;
   p.open0 = g.open[1];
@@ -371,7 +373,9 @@ int tile2d_step(const Grid& g, const Opts& o, const StepArgs<T>& a, int fields, 
   p.rhs_a = o.rhs_a;
   p.rhs_b = o.rhs_b;
   p.chained = a.chained;
-#define MPD_T(F, I) (o.nug ? launch_tile<T, F, I, true>(p, fields, st) : launch_tile<T, F, I, false>(p, fields, st))
+  const bool always = o.kernel != 0;  // MPDATA_TUNE_KERNEL asks for a fused kernel
+#define MPD_T(F, I) \
+  (o.nug ? launch_tile<T, F, I, true>(p, fields, always, st) : launch_tile<T, F, I, false>(p, fields, always, st))
   if (o.fct) return o.iga ? MPD_T(true, true) : MPD_T(true, false);
   return o.iga ? MPD_T(false, true) : MPD_T(false, false);
 #undef MPD_T

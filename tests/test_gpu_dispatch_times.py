@@ -55,3 +55,15 @@ def test_fp64_ensembles_take_a_tile_height_near_the_best(shapes):
     rows = (0, 12, 16, 24, 32, 48)
     got = times(*[problem(shapes, torch.float64, 2, capi.FCT, {capi.TUNE_TILE_ROWS: r}) for r in rows])
     assert got[0] <= 1.1 * min(got[1:]), dict(zip(rows, got))
+
+
+@pytest.mark.parametrize("n,dtype,n_iters,opts", [
+    (64, torch.float64, 3, capi.FCT), (64, torch.float64, 8, capi.FCT), (64, torch.float64, 3, 0),
+    (256, torch.float64, 6, capi.FCT), (512, torch.float64, 5, capi.TOT), (1024, torch.float64, 3, capi.TOT | capi.FCT),
+    (1024, torch.float64, 3, 0), (1024, torch.float64, 2, capi.TOT), (64, torch.float32, 8, capi.TOT | capi.FCT),
+    (512, torch.float32, 6, capi.FCT), (1024, torch.float32, 8, capi.FCT), (1024, torch.float32, 3, capi.FCT)])
+def test_steps_beyond_two_passes_take_the_better_kernels(n, dtype, n_iters, opts):
+    auto, tile, staged = times(problem((n, n), dtype, n_iters, opts),
+                               problem((n, n), dtype, n_iters, opts, {capi.TUNE_KERNEL: 1}),
+                               problem((n, n), dtype, n_iters, opts | capi.STAGED))
+    assert auto <= 1.15 * min(tile, staged), (auto, tile, staged)
