@@ -135,7 +135,7 @@ def measured_peaks():
 
 
 KERNEL_NAMES = {1: "k_fused2d", 2: "k_band2d", 3: "k_fused2d_nc2"}
-_WARP_MARCH = ("fused2d.cu", "march2d.cuh", "stencil2d.cuh")
+_WARP_MARCH = ("fused2d.cu", "march2d.cuh", "lanes2d.h", "stencil2d.cuh")
 KERNEL_SOURCES = {"k_fused2d": _WARP_MARCH, "k_band2d": ("band2d.cu", "stencil2d.cuh"), "k_fused2d_comp": _WARP_MARCH,
                   "k_fused2d_nc2": _WARP_MARCH, "k_fused2d_comp_nc2": _WARP_MARCH}
 

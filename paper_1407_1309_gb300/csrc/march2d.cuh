@@ -26,6 +26,7 @@
 #include <type_traits>
 
 #include "kernels.h"
+#include "lanes2d.h"
 #include "launch.cuh"
 #include "stencil2d.cuh"
 
@@ -34,18 +35,16 @@ namespace {
 
 using namespace dev;
 
-constexpr int kLead = 4;     // computed columns left of the strip's first output column
 constexpr int kPF = 4;       // rows in flight
 constexpr int kSlots = kPF + 1;
 // arrays in a ring slot: psi, gc0, gc1, G, R [, lo of the compensated state]
 template <bool COMP> constexpr int arrs() { return COMP ? 6 : 5; }
-constexpr int kWarps = 4;    // warps per block
 
 // EXT bits: |psi| in the psi-fractions (Sect. 3.1.5), the divergent-flow term (Sect. 3.1.3)
 constexpr int kExtAbs = 1, kExtDfl = 2;
 
 template <int NC> constexpr int cols() { return 32 * NC; }
-template <int NC> constexpr int stride() { return 32 * NC - 2 * kLead; }
+template <int NC> constexpr int stride() { return strip_stride(NC); }
 
 template <typename T>
 struct F2Params {
@@ -467,49 +466,6 @@ void launch(const F2Params<T>& p, cudaStream_t st) {
 
 inline bool al(const void* q, size_t a) { return q == nullptr || (reinterpret_cast<uintptr_t>(q) % a) == 0; }
 
-// Tile height of the FP32 warp march and the time it should take.  Every warp of a tile height ty
-// marches ty + 6 rows; with k blocks on the fullest SM one row of all of them takes it c(k)
-// microseconds, more than k times one block's share only while few warps leave the issue slots idle
-// (c measured on fields of 256^2 .. 4096^2: one block takes almost as long as two; three of the
-// plain march with lanes of 4 fit an SM at once).  The height is the smallest that keeps the fullest
-// SM at k blocks, for the k of least time.  Against the earlier list of heights (the tallest with
-// 7.5 warps per SM): 4096^2 102 -> 89 us (79 rows instead of 64), 2000 x 500 13.9 -> 10.8 us (with
-// lanes of 2).
-struct MarchRows {
-  int ty;
-  float us;
-};
-template <int NC>
-inline MarchRows march_rows(int n0, int n1, bool comp) {
-  static_assert(NC == 4 || NC == 2, "lanes of 4 or 2 columns");
-  static const float plain4[4] = {0.55f, 0.73f, 1.00f, 1.44f}, plain2[4] = {0.38f, 0.455f, 0.59f, 0.74f};
-  static const float comp4[4] = {0.93f, 0.97f, 1.37f, 1.83f}, comp2[4] = {0.53f, 0.58f, 0.76f, 0.97f};
-  const float* c = NC == 4 ? (comp ? comp4 : plain4) : (comp ? comp2 : plain2);
-  const long long strips = (n1 + stride<NC>() - 1) / stride<NC>();
-  constexpr long long kSms = 152;
-  MarchRows best{n0 > 4 ? n0 : 4, 0.0f};
-  bool any = false;
-  for (long long k = 1; k <= 6; ++k) {
-    const long long tiles = kSms * k * kWarps / strips;
-    if (tiles < 1) continue;
-    long long ty = (n0 + tiles - 1) / tiles;
-    if (ty < 4) ty = 4;
-    const long long blocks = (strips * ((n0 + ty - 1) / ty) + kWarps - 1) / kWarps;
-    const long long full = (blocks + kSms - 1) / kSms;
-    const float us = static_cast<float>(ty + 6) * (full <= 4 ? c[full - 1] : c[2] / 3.0f * static_cast<float>(full));
-    if (!any || us < best.us) best = {static_cast<int>(ty), us};
-    any = true;
-  }
-  return best;
-}
-
-// Whether lanes of 2 columns suit an FP32 field better than lanes of 4: where the narrower strips
-// leave fewer padded columns or, on a field too small to fill the GPU, their twice as many warps
-// hide more latency (compensated 512^2 12.1 -> 8.1 us, plain 2000 x 500 13.9 -> 10.8).
-inline bool narrow_lanes(int n0, int n1, bool comp) {
-  return march_rows<2>(n0, n1, comp).us < 0.98f * march_rows<4>(n0, n1, comp).us;
-}
-
 // Warp-march parameters of one step of one field; *band is set when the automatic choice is
 // the band march.  NC columns per lane: FP32 lanes own 4 (16-byte copies) or 2 (narrow_lanes, or
 // MPDATA_TUNE_KERNEL = 3), FP64 lanes 2 (register budget).
@@ -528,7 +484,7 @@ F2Params<T> warp_params(const Grid& g, const Opts& o, const StepArgs<T>& a, bool
   auto warps = [&](int ty) { return static_cast<long long>(p.strips) * ((p.n0 + ty - 1) / ty); };
   int auto_ty = 8;
   if constexpr (sizeof(T) == 4) {
-    auto_ty = march_rows<NC>(p.n0, p.n1, comp).ty;
+    auto_ty = march_rows(NC, p.n0, p.n1, comp).ty;
   } else {  // FP64: the tallest tile that still gives ~7.5 warps per SM (152 SMs), at least 8 rows
     for (int ty : {64, 48, 32, 24, 16, 12}) {
       if (warps(ty) >= 1140) { auto_ty = ty; break; }
