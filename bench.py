@@ -690,7 +690,7 @@ def bench_config1(dev):
     return {"workload": "1d_box_gaussian_n500_c0.5_n_iters2_f64", "steps": 1000, "time_ms": round(secs * 1e3, 3),
             "value": round(500 * 1000 / secs / 1e9, 4), "unit": UNIT,
             "one_transit_rms_err_vs_initial": float(np.sqrt(np.mean((out - psi) ** 2))),
-            "path": "one launch of one thread-block cluster for all steps (field in registers, halos through distributed "
+            "path": "one thread-block cluster, 256 steps per launch (field in registers, halos through distributed "
                     "shared memory)"}
 
 

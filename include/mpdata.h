@@ -155,8 +155,8 @@ int mpdata_sw_reset(mpdata_t h);
  * 2D steps run fused kernels (one launch per step; more than two passes, the third-order terms and
  * open edges as a shared-memory tile kernel where that should be faster than one kernel per
  * sub-step, MPDATA_TUNE_KERNEL), 1D fields short enough for
- * one thread-block cluster (about 10000 cells with two passes) run the whole call in one launch,
- * and so do such 1D systems with trapezoidal sources; the rest run one kernel per sub-step.
+ * one thread-block cluster (about 10000 cells with two passes), and such 1D systems with
+ * trapezoidal sources, run 256 steps per launch; the rest run one kernel per sub-step.
  * gc (host array of ndims device pointers): advector components, constant over
  * the call.  g: G field (required iff MPDATA_NUG, else NULL).  r: source term R
  * (required iff an RHS bit is set, else NULL), dt its time step.
@@ -284,8 +284,9 @@ int mpdata_check_courant(mpdata_t h, const void* const* gc, const void* g, doubl
  * Asks the handle to stop: later mpdata_step / mpdata_advance calls return
  * MPDATA_ESTOPPED without enqueuing work, and a multi-step call stops after the
  * step in progress (the paper's panic flag, Sect. 3.2.5).  A 1D field (or 1D system with
- * trapezoidal sources) short enough for one cluster runs every step of a call in one launch; for
- * it the request takes effect at the next call.  Thread-safe.  mpdata_clear_stop
+ * trapezoidal sources) short enough for one cluster runs 256 steps per launch and stops after those;
+ * one of up to 2235 (FP64) / 4470 (FP32) cells with more passes than the cluster takes runs every
+ * step of a call in one launch, and the request takes effect at the next call.  Thread-safe.  mpdata_clear_stop
  * re-arms the handle.
  */
 int mpdata_request_stop(mpdata_t h);

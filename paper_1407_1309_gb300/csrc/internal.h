@@ -171,14 +171,15 @@ struct TrapezMat {
 // Minv of I - dt/2 A by Gauss-Jordan elimination with partial pivoting; false if singular.
 bool trapez_matrix(TrapezMat& m, const double* A, int E, double dt);
 
-// Every step of a call for a 1D field, or (m not null: its matrices and b) for a system of m->E 1D
+// n_steps steps of a 1D field, or (m not null: its matrices and b) of a system of m->E 1D
 // equations of g.N cells each with trapezoidal sources, in one launch of one thread-block cluster
 // (line1d.cu): the field in registers, halos exchanged through distributed shared memory.
 // MPDATA_EUNSUPPORTED (nothing launched) for the divergent-flow term, open edges, FP64 |psi|, steps
-// that reach more than 12 cells and fields too long for one cluster.
+// that reach more than 12 cells and fields too long for one cluster.  chained: as a dependent of the
+// kernel before it (launch.cuh).
 template <typename T>
 int line1d_steps(const Grid& g, const Opts& o, const T* psi_in, T* psi_out, const T* gc, const T* G, const T* R, T dt,
-                 int n_steps, const TrapezMat* m, const T* b, cudaStream_t st);
+                 int n_steps, const TrapezMat* m, const T* b, bool chained, cudaStream_t st);
 
 // Intermediates of one forward step kept for the adjoint (n_iters <= kTapeMax).
 constexpr int kTapeMax = 4;

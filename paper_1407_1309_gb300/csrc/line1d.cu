@@ -1,5 +1,5 @@
-// Every step of a call for a 1D field, or for a system of 1D equations with trapezoidal sources
-// (Sect. 4.1), in one launch of one thread-block cluster.
+// Many steps of a 1D field, or of a system of 1D equations with trapezoidal sources (Sect. 4.1), in
+// one launch of one thread-block cluster.
 //
 // What bounds it: a 1D field of the usual size (100 .. 2000 cells) is too small to fill the GPU and
 // its steps depend on each other, so the call costs n_steps times the latency of one step.  One
@@ -30,6 +30,7 @@
 #include <cuda_runtime.h>
 
 #include "internal.h"
+#include "launch.cuh"
 #include "stencil2d.cuh"
 
 namespace mpd {
@@ -219,6 +220,8 @@ __global__ void __launch_bounds__(32 * kMaxWarps) k_line1d(const LineParams<T> p
     }
   };
 
+  // the launch before this one, when launched as its dependent; it wrote psi, not what is read above
+  grid_wait();
   T q;
   T x[kTrapezMax];
   if (SYS) {
@@ -295,7 +298,7 @@ int largest_cluster() {
 }
 
 template <typename T, bool FCT, bool IGA, bool SYS>
-int launch_line(LineParams<T> p, cudaStream_t st) {
+int launch_line(LineParams<T> p, bool chained, cudaStream_t st) {
   const int room = 32 - 2 * p.halo;  // cells of its own per warp, one step between exchanges
   if (room < kLeast) return MPDATA_EUNSUPPORTED;
   // the smallest cluster that gives every warp's SM one chunk per equation (more blocks only add
@@ -319,12 +322,14 @@ int launch_line(LineParams<T> p, cudaStream_t st) {
   cfg.blockDim = dim3(static_cast<unsigned>(32 * p.chunks * p.E));
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = static_cast<unsigned>(C);
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = chained ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, k_line1d<T, FCT, IGA, SYS>, p) == cudaSuccess ? MPDATA_OK : MPDATA_ECUDA;
 }
 
@@ -332,7 +337,7 @@ int launch_line(LineParams<T> p, cudaStream_t st) {
 
 template <typename T>
 int line1d_steps(const Grid& g, const Opts& o, const T* psi_in, T* psi_out, const T* gc, const T* G, const T* R, T dt,
-                 int n_steps, const TrapezMat* m, const T* b, cudaStream_t st) {
+                 int n_steps, const TrapezMat* m, const T* b, bool chained, cudaStream_t st) {
   if (g.nd != 1 || o.dfl || o.open) return MPDATA_EUNSUPPORTED;
   // FP64 |psi| stays on the staged kernels: on a positive field it is their basic scheme bit for bit
   if (o.abs && sizeof(T) == 8) return MPDATA_EUNSUPPORTED;
@@ -360,16 +365,16 @@ int line1d_steps(const Grid& g, const Opts& o, const T* psi_in, T* psi_out, cons
   p.dt = dt;
   if (m) {
     p.m = *m;
-    if (o.fct) return o.iga ? launch_line<T, true, true, true>(p, st) : launch_line<T, true, false, true>(p, st);
-    return o.iga ? launch_line<T, false, true, true>(p, st) : launch_line<T, false, false, true>(p, st);
+    if (o.fct) return o.iga ? launch_line<T, true, true, true>(p, chained, st) : launch_line<T, true, false, true>(p, chained, st);
+    return o.iga ? launch_line<T, false, true, true>(p, chained, st) : launch_line<T, false, false, true>(p, chained, st);
   }
-  if (o.fct) return o.iga ? launch_line<T, true, true, false>(p, st) : launch_line<T, true, false, false>(p, st);
-  return o.iga ? launch_line<T, false, true, false>(p, st) : launch_line<T, false, false, false>(p, st);
+  if (o.fct) return o.iga ? launch_line<T, true, true, false>(p, chained, st) : launch_line<T, true, false, false>(p, chained, st);
+  return o.iga ? launch_line<T, false, true, false>(p, chained, st) : launch_line<T, false, false, false>(p, chained, st);
 }
 
 template int line1d_steps<float>(const Grid&, const Opts&, const float*, float*, const float*, const float*,
-                                 const float*, float, int, const TrapezMat*, const float*, cudaStream_t);
+                                 const float*, float, int, const TrapezMat*, const float*, bool, cudaStream_t);
 template int line1d_steps<double>(const Grid&, const Opts&, const double*, double*, const double*, const double*,
-                                  const double*, double, int, const TrapezMat*, const double*, cudaStream_t);
+                                  const double*, double, int, const TrapezMat*, const double*, bool, cudaStream_t);
 
 }  // namespace mpd
