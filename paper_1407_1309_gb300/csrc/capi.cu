@@ -24,6 +24,7 @@ struct mpdata_s {
   void* pingpong = nullptr;          // out-of-place buffer for the fused paths (total elements)
   void* pingpong_lo = nullptr;       // its low-part twin for the compensated state (on first use)
   void* adj = nullptr;               // adjoint scratch
+  bool adj_released = false;         // the last reverse sweep releases its successor early
   mpd::FieldSpan* d_spans = nullptr;
   double* d_partial = nullptr;       // 2 * kRedBlocks * n_fields
   double* d_out = nullptr;           // 2 * n_fields
@@ -259,6 +260,7 @@ cudaStream_t handle_stream(const mpdata_s* h) { return h->stream; }
 int* handle_status(const mpdata_s* h) { return h->d_status; }
 void** handle_batch(mpdata_s* h) { return &h->batch; }
 void** handle_adj(mpdata_s* h) { return &h->adj; }
+bool* handle_adj_released(mpdata_s* h) { return &h->adj_released; }
 int handle_n_iters(const mpdata_s* h) { return h->n_iters; }
 uint32_t handle_opts(const mpdata_s* h) { return h->opts; }
 void handle_tuning(const mpdata_s* h, int* kernel, int* tile_rows) {

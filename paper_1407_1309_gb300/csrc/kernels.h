@@ -15,6 +15,8 @@ cudaStream_t handle_stream(const mpdata_s* h);
 int* handle_status(const mpdata_s* h);
 void** handle_batch(mpdata_s* h);
 void** handle_adj(mpdata_s* h);
+// whether the handle's last reverse sweep releases its successor early (adjoint.cu)
+bool* handle_adj_released(mpdata_s* h);
 int handle_n_iters(const mpdata_s* h);
 uint32_t handle_opts(const mpdata_s* h);
 // the handle's MPDATA_TUNE_KERNEL and MPDATA_TUNE_TILE_ROWS settings

@@ -67,3 +67,33 @@ def test_steps_beyond_two_passes_take_the_better_kernels(n, dtype, n_iters, opts
                                problem((n, n), dtype, n_iters, opts, {capi.TUNE_KERNEL: 1}),
                                problem((n, n), dtype, n_iters, opts | capi.STAGED))
     assert auto <= 1.15 * min(tile, staged), (auto, tile, staged)
+
+
+@pytest.mark.parametrize("pair", [False, True], ids=["one_call", "record_and_replay"])
+def test_reverse_step_takes_no_longer_than_its_parts(pair):
+    """1024^2 FP32 with the limiter, 20 reverse steps, each in one call or as a recording and a replay,
+    against 20 recordings and then 20 replays."""
+    n, steps = 1024, 20
+    gen = torch.Generator(device=DEV).manual_seed(2)
+    psi = 2 + torch.rand((n, n), generator=gen, device=DEV)
+    gc = [0.4 * (torch.rand((n, n), generator=gen, device=DEV) - 0.5) for _ in range(2)]
+    nxt, pb, gcb = torch.empty_like(psi), torch.rand((n, n), generator=gen, device=DEV), [torch.zeros_like(v) for v in gc]
+    m = Mpdata((n, n), dtype=torch.float32, n_iters=2, opts=capi.FCT)
+    tape = torch.empty(m.tape_numel(), device=DEV)
+
+    def whole():
+        for _ in range(steps):
+            if pair:
+                m.adjoint_record(psi, gc, tape, psi_next=nxt)
+                m.adjoint_replay(psi, gc, tape, pb, gc_bar=gcb)
+            else:
+                m.adjoint_step(psi, gc, pb, gc_bar=gcb)
+
+    def parts():
+        for _ in range(steps):
+            m.adjoint_record(psi, gc, tape, psi_next=nxt)
+        for _ in range(steps):
+            m.adjoint_replay(psi, gc, tape, pb, gc_bar=gcb)
+
+    one, two = times(whole, parts)
+    assert one <= 1.08 * two, (one, two)
