@@ -97,3 +97,11 @@ def test_reverse_step_takes_no_longer_than_its_parts(pair):
 
     one, two = times(whole, parts)
     assert one <= 1.08 * two, (one, two)
+
+
+def test_wide_fields_take_a_tile_height_near_the_best():
+    """1250 strips: whole tiles per SM leave few heights to choose from."""
+    rows = (0, 32, 64)
+    got = times(*[problem((1500, 150000), torch.float32, 2, capi.FCT,
+                          {capi.TUNE_TILE_ROWS: r, capi.TUNE_KERNEL: 1} if r else {}) for r in rows])
+    assert got[0] <= 1.08 * min(got[1:]), dict(zip(rows, got))
