@@ -207,8 +207,8 @@ template <typename T>
 cudaError_t trapez_post(const TrapezMat& m, long long n, T dt, const T* b, T* psi, bool chained, cudaStream_t st);
 
 // Vectorised FP32 pseudo-advector z-march for 3D fields (march3.cu): launched, and true
-// returned, when the x extent is at least 48 and no edge is open; false (nothing launched)
-// otherwise.  chained: as a dependent of the kernel before it (launch.cuh).
+// returned, when no edge is open, the x extent is at least 48 and the field large enough that it
+// is the faster form (march3_form); false (nothing launched) otherwise.  chained: as a dependent of the kernel before it (launch.cuh).
 bool antidiff3_vec(const Grid& g, const float* psi, const float* const* v, float vscale, const float* G, bool iga,
                    bool tot, bool abs_psi, float* const* out, bool chained, cudaStream_t st);
 

@@ -22,6 +22,7 @@
 
 #include "internal.h"
 #include "launch.cuh"
+#include "march3_cost.h"
 #include "stencil2d.cuh"
 
 namespace mpd {
@@ -29,7 +30,7 @@ namespace {
 
 using namespace dev;
 
-constexpr int kRows = 8;     // tile rows, one warp each
+constexpr int kRows = kMarchRows;  // tile rows, one warp each
 constexpr int kThreads = 32 * kRows;
 template <int NC> constexpr int row_w() { return 32 * NC + 8; }  // row with 4 halo cells each side
 
@@ -905,27 +906,6 @@ inline dim3 march_grid(const Grid& g, int zc) {
               static_cast<unsigned>((g.n[1] + kRows - 1) / kRows), static_cast<unsigned>((g.n[0] + zc - 1) / zc));
 }
 
-// z-planes per block, 4 to 16: the chunk of least time by the load of the fullest SM.  A block takes
-// about zc + 3 plane steps (its halo planes are staged, pass 1 and the factors recomputed on two of
-// them); two blocks share an SM and take 1.5 times as long as one there.  Large fields get 16
-// (measured at 256^3: 8 .. 24 within 2 %); 128^3, one block per SM with 16, gets 7 and two: 206 -> 151
-// us per step of three passes with third-order terms.
-template <int NC>
-inline int z_chunk(const Grid& g) {
-  int best = 16;
-  float least = 0.0f;
-  for (int zc = 16; zc >= 4; --zc) {
-    const dim3 b = march_grid<NC>(g, zc);
-    const long long k = (static_cast<long long>(b.x) * b.y * b.z + 151) / 152;
-    const float t = static_cast<float>(zc + 3) * (k == 1 ? 1.0f : 0.75f * static_cast<float>(k));
-    if (zc == 16 || t < 0.98f * least) {
-      best = zc;
-      least = t;
-    }
-  }
-  return best;
-}
-
 // The chunk of large fields is a compile-time constant (a run-time one made the pseudo-advector of
 // 256^3 cells 236 instead of 226 us, at the same registers).
 template <bool VEC, class F>
@@ -948,7 +928,7 @@ inline void want_smem(PerDevice<bool>& attr, K kern, size_t bytes) {
 template <int NC, int MINB, bool VEC, bool ABS, bool IGA, bool TOT, bool NUG>
 void launch_v(const Grid& g, const float* psi, const float* const* v, float vscale, const float* G, float* const* out,
               bool chained, cudaStream_t st) {
-  const int zc = z_chunk<NC>(g);
+  const int zc = z_chunk(g.n, NC).zc;
   V3 vin{{v[0], v[1], v[2]}};
   O3 vo{{out[0], out[1], out[2]}};
   with_chunk<VEC>(zc, [&](auto c) {
@@ -962,7 +942,7 @@ void launch_v(const Grid& g, const float* psi, const float* const* v, float vsca
 template <int NC, bool VEC, bool KAHAN, bool NUG>
 void launch_b(const Grid& g, const float* psi, const float* const* v, float vscale, const float* G, float* p1,
               float* mx, float* mn, bool chained, cudaStream_t st) {
-  const int zc = z_chunk<NC>(g);
+  const int zc = z_chunk(g.n, NC).zc;
   V3 vv{{v[0], v[1], v[2]}};
   with_chunk<VEC>(zc, [&](auto c) {
     auto kern = k_p1b3v<NC, VEC, decltype(c)::value, KAHAN, NUG>;
@@ -975,7 +955,7 @@ void launch_b(const Grid& g, const float* psi, const float* const* v, float vsca
 template <int NC, bool VEC, bool NUG, bool UNIT, bool LIM>
 void launch_k(const Grid& g, const float* psi, const float* const* vu, const float* G, const float* mx,
               const float* mn, float* const* lim, float* out, bool chained, cudaStream_t st) {
-  const int zc = z_chunk<NC>(g);
+  const int zc = z_chunk(g.n, NC).zc;
   V3 vv{{vu[0], vu[1], vu[2]}};
   O3 lo{{lim[0], lim[1], lim[2]}};
   with_chunk<VEC>(zc, [&](auto c) {
@@ -1029,12 +1009,12 @@ void corr3_nc(const Grid& g, const float* psi, const float* const* vu, const flo
 
 }  // namespace
 
-// The forms for fields whose rows cannot be moved in 16-byte chunks (march3u.cu).
-void antidiff3_cells(const Grid& g, const float* psi, const float* const* v, float vscale, const float* G, bool iga,
-                     bool tot, bool abs_psi, float* const* out, bool chained, cudaStream_t st);
-void p1b3_cells(const Grid& g, const float* psi, const float* const* v, float vscale, const float* G, bool kahan,
+// The forms staged cell by cell (march3u.cu), with lanes of 2 cells or of 4.
+void antidiff3_cells(const Grid& g, bool two, const float* psi, const float* const* v, float vscale, const float* G,
+                     bool iga, bool tot, bool abs_psi, float* const* out, bool chained, cudaStream_t st);
+void p1b3_cells(const Grid& g, bool two, const float* psi, const float* const* v, float vscale, const float* G, bool kahan,
                 float* p1, float* mx, float* mn, bool chained, cudaStream_t st);
-void corr3_cells(const Grid& g, const float* psi, const float* const* vu, const float* G, bool iga, const float* mx,
-                 const float* mn, float* const* lim, float* out, bool chained, cudaStream_t st);
+void corr3_cells(const Grid& g, bool two, const float* psi, const float* const* vu, const float* G, bool iga,
+                 const float* mx, const float* mn, float* const* lim, float* out, bool chained, cudaStream_t st);
 
 }  // namespace mpd

@@ -2,7 +2,7 @@
 // chunks (x extents that are no multiple of 4, unaligned arrays) and for fields of fewer than 128
 // columns: the planes are staged cell by cell (4-byte cp.async, each cell wrapped by itself), the
 // arithmetic on the staged rows is the same.  Lanes of 4 or of 2 cells (tiles of 128 or 64
-// columns), whichever pads the rows less.
+// columns; march3_form).
 //
 // Against the scalar z-marches of staged.cu, whose threads own one cell each: 101 x 97 x 103 with
 // three passes, third-order terms, limiter and G 233 -> 149 us per step, 64^3 133 -> 59,
@@ -10,32 +10,22 @@
 #include "march3.cuh"
 
 namespace mpd {
-namespace {
 
-// lanes of 2 cells where 64-column tiles cover the row with at most 3/4 of the columns that
-// 128-column tiles compute
-bool narrow(const Grid& g) {
-  const int w4 = (g.n[2] + 127) / 128 * 128, w2 = (g.n[2] + 63) / 64 * 64;
-  return 4 * w2 <= 3 * w4;
-}
-
-}  // namespace
-
-void antidiff3_cells(const Grid& g, const float* psi, const float* const* v, float vscale, const float* G, bool iga,
-                     bool tot, bool abs_psi, float* const* out, bool chained, cudaStream_t st) {
-  if (narrow(g)) antidiff3_nc<2, false>(g, psi, v, vscale, G, iga, tot, abs_psi, out, chained, st);
+void antidiff3_cells(const Grid& g, bool two, const float* psi, const float* const* v, float vscale, const float* G,
+                     bool iga, bool tot, bool abs_psi, float* const* out, bool chained, cudaStream_t st) {
+  if (two) antidiff3_nc<2, false>(g, psi, v, vscale, G, iga, tot, abs_psi, out, chained, st);
   else antidiff3_nc<4, false>(g, psi, v, vscale, G, iga, tot, abs_psi, out, chained, st);
 }
 
-void p1b3_cells(const Grid& g, const float* psi, const float* const* v, float vscale, const float* G, bool kahan,
+void p1b3_cells(const Grid& g, bool two, const float* psi, const float* const* v, float vscale, const float* G, bool kahan,
                 float* p1, float* mx, float* mn, bool chained, cudaStream_t st) {
-  if (narrow(g)) p1b3_nc<2, false>(g, psi, v, vscale, G, kahan, p1, mx, mn, chained, st);
+  if (two) p1b3_nc<2, false>(g, psi, v, vscale, G, kahan, p1, mx, mn, chained, st);
   else p1b3_nc<4, false>(g, psi, v, vscale, G, kahan, p1, mx, mn, chained, st);
 }
 
-void corr3_cells(const Grid& g, const float* psi, const float* const* vu, const float* G, bool iga, const float* mx,
-                 const float* mn, float* const* lim, float* out, bool chained, cudaStream_t st) {
-  if (narrow(g)) corr3_nc<2, false>(g, psi, vu, G, iga, mx, mn, lim, out, chained, st);
+void corr3_cells(const Grid& g, bool two, const float* psi, const float* const* vu, const float* G, bool iga,
+                 const float* mx, const float* mn, float* const* lim, float* out, bool chained, cudaStream_t st) {
+  if (two) corr3_nc<2, false>(g, psi, vu, G, iga, mx, mn, lim, out, chained, st);
   else corr3_nc<4, false>(g, psi, vu, G, iga, mx, mn, lim, out, chained, st);
 }
 

@@ -27,6 +27,16 @@ def problem(shapes, dtype, n_iters, opts, knobs=None):
     return lambda: m.advance(psi, out, gc, n_steps=4)
 
 
+def problem3(shape):
+    """A call of 4 limited two-pass steps of a random 3D FP32 field, ready to be timed."""
+    gen = torch.Generator(device=DEV).manual_seed(1)
+    psi = 2 + torch.rand(shape, generator=gen, device=DEV)
+    gc = [0.3 * (torch.rand(shape, generator=gen, device=DEV) - 0.5) for _ in range(3)]
+    out = torch.empty_like(psi)
+    m = Mpdata(shape, dtype=torch.float32, n_iters=2, opts=capi.FCT)
+    return lambda: m.advance(psi, out, gc, n_steps=4)
+
+
 def times(*calls):
     """Median microseconds of each call, timed in turn."""
     got = [[] for _ in calls]
