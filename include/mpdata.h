@@ -155,7 +155,7 @@ int mpdata_sw_reset(mpdata_t h);
  * 2D steps run fused kernels (one launch per step; more than two passes, the third-order terms and
  * open edges as a shared-memory tile kernel where that should be faster than one kernel per
  * sub-step, MPDATA_TUNE_KERNEL), 1D fields short enough for
- * one thread-block cluster (about 10000 cells with two passes), and such 1D systems with
+ * one thread-block cluster (about 10000 cells with two passes, fewer in FP64 with more), and such 1D systems with
  * trapezoidal sources, run 256 steps per launch; the rest run one kernel per sub-step.
  * gc (host array of ndims device pointers): advector components, constant over
  * the call.  g: G field (required iff MPDATA_NUG, else NULL).  r: source term R

@@ -175,7 +175,8 @@ bool trapez_matrix(TrapezMat& m, const double* A, int E, double dt);
 // equations of g.N cells each with trapezoidal sources, in one launch of one thread-block cluster
 // (line1d.cu): the field in registers, halos exchanged through distributed shared memory.
 // MPDATA_EUNSUPPORTED (nothing launched) for the divergent-flow term, open edges, FP64 |psi|, steps
-// that reach more than 12 cells and fields too long for one cluster.  chained: as a dependent of the
+// that reach more than 12 cells, fields too long for one cluster and FP64 fields long enough that the
+// staged kernels are faster.  chained: as a dependent of the
 // kernel before it (launch.cuh).
 template <typename T>
 int line1d_steps(const Grid& g, const Opts& o, const T* psi_in, T* psi_out, const T* gc, const T* G, const T* R, T dt,

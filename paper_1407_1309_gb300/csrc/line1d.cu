@@ -309,6 +309,16 @@ int launch_line(LineParams<T> p, bool chained, cudaStream_t st) {
   const int most = (p.n + C - 1) / C;
   p.chunks = (most + room - 1) / room;
   if (p.chunks * p.E > kMaxWarps) return MPDATA_EUNSUPPORTED;
+  // An FP64 field of many chunks per SM waits for the cluster's FP64 pipes, and the launches of the
+  // staged kernels, spread over all SMs, take less: microseconds per step of either, fitted to 50 ..
+  // 12000 cells and 1 .. 6 passes (K4 with third-order terms and limiter, 4000 cells 36.7 and 36.4,
+  // 6000 cells 55 and 37; two passes with the limiter 10000 cells 10.8 and 12.7).  Systems, whose
+  // staged form takes the launches of every equation, and FP32 are faster here at every length.
+  if (sizeof(T) == 8 && !SYS) {
+    const double passes = p.K - 1, fct = FCT ? 1.0 : 0.0, tot = p.tot ? 1.0 : 0.0;
+    const double here = p.chunks * (0.09 + passes * (0.2 + 0.145 * fct + 0.2 * tot));
+    if (here > 1.8 + passes * (4.75 + 5.2 * fct + 1.9 * tot)) return MPDATA_EUNSUPPORTED;
+  }
   const int u = (most + p.chunks - 1) / p.chunks;
   p.S = 1;
   if (!SYS) {

@@ -115,3 +115,19 @@ def test_wide_fields_take_a_tile_height_near_the_best():
     got = times(*[problem((1500, 150000), torch.float32, 2, capi.FCT,
                           {capi.TUNE_TILE_ROWS: r, capi.TUNE_KERNEL: 1} if r else {}) for r in rows])
     assert got[0] <= 1.08 * min(got[1:]), dict(zip(rows, got))
+
+
+@pytest.mark.parametrize("n,n_iters,opts", [(6000, 4, capi.TOT | capi.FCT), (8000, 3, capi.TOT | capi.FCT), (12000, 2, 0),
+                                            (4000, 2, capi.FCT)])
+def test_long_fp64_lines_take_the_better_kernels(n, n_iters, opts):
+    gen = torch.Generator(device=DEV).manual_seed(3)
+    psi = 2 + torch.rand(n, generator=gen, device=DEV, dtype=torch.float64)
+    gc = [torch.full((n,), 0.3, device=DEV, dtype=torch.float64)]
+    out = torch.empty_like(psi)
+
+    def steps(extra):
+        m = Mpdata((n,), dtype=torch.float64, n_iters=n_iters, opts=opts | extra)
+        return lambda: m.advance(psi, out, gc, n_steps=40)
+
+    auto, staged = times(steps(0), steps(capi.STAGED))
+    assert auto <= 1.15 * staged, (auto, staged)
