@@ -14,9 +14,10 @@ constexpr int strip_stride(int nc) { return 32 * nc - 2 * kLead; }
 // microseconds, more than k times one block's share only while few warps leave the issue slots idle
 // (c measured on fields of 256^2 .. 4096^2: one block takes almost as long as two; three of the
 // plain march with lanes of 4 fit an SM at once).  The height is the smallest that keeps the fullest
-// SM at k blocks, for the k of least time; a field with more strips than that has warps is not cut
-// into rows.  Against the earlier list of heights (the tallest with 7.5 warps per SM): 4096^2
-// 102 -> 89 us (79 rows instead of 64), 2000 x 500 13.9 -> 10.8 us (with lanes of 2).
+// SM at k blocks, for the k of least time, even (the march's loop takes two rows a turn, and its
+// single last row of an odd height rounds the products differently, so that a result would depend
+// on the height); a field with more strips than that has warps is not cut into rows.  Against the earlier list of heights (the tallest with 7.5 warps per SM): 4096^2
+// 102 -> 90 us (80 rows instead of 64), 2000 x 500 13.9 -> 10.8 us (with lanes of 2).
 struct MarchRows {
   int ty;
   float us;
@@ -35,6 +36,7 @@ inline MarchRows march_rows(int nc, int n0, int n1, bool comp) {
     const long long tiles = kSms * k * kWarps / strips;
     long long ty = tiles < 1 ? n0 : (n0 + tiles - 1) / tiles;
     if (ty < 4) ty = 4;
+    ty += ty & 1;
     const long long blocks = (strips * ((n0 + ty - 1) / ty) + kWarps - 1) / kWarps;
     const long long full = (blocks + kSms - 1) / kSms;
     const float us = static_cast<float>(ty + 6) * (full <= 4 ? c[full - 1] : c[2] / 3.0f * static_cast<float>(full));
