@@ -35,10 +35,10 @@
  * asynchronous; a device-side failure is reported by the next call on the
  * handle that synchronises (mpdata_reduce, mpdata_sync).  The blocks of a grid
  * wait for each other only inside one thread-block cluster, whose blocks the
- * hardware runs at the same time (the 1D path's cluster barrier); the reverse
- * step's kernels, launched as programmatic dependents, wait only for the
- * completion of the kernel before them on the stream.  No call can hang on a
- * device-side wait.
+ * hardware runs at the same time (the 1D path's cluster barrier).  The kernels of
+ * a call after its first, and the reverse step's, are launched as programmatic
+ * dependents and wait only for the completion of the kernel before them on the
+ * stream.  No call can hang on a device-side wait.
  */
 #ifndef MPDATA_GB300_H
 #define MPDATA_GB300_H

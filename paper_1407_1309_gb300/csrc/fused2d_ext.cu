@@ -2,9 +2,9 @@
 // Sect. 3.1.5), the divergent-flow term (Sect. 3.1.3) or both: a translation unit of its own
 // beside fused2d.cu so that the two compile side by side.
 //
-// Bound by issue like the plain march, whose instructions these options barely add to (|x| is an
-// operand modifier; the divergence takes four adds per cell and two fma per face).  Measured: |psi| with the limiter on
-// 1021 x 1000 cells 80.3 us per step on the staged kernels, 12.3 us here.
+// Bound by issue like the plain march, whose instructions these options barely add to (the
+// divergence takes four adds per cell and two fma per face).  Measured: |psi| with the limiter on
+// 1021 x 1000 cells 80.3 us per step on the staged kernels, 11.3 us here.
 #include "march2d.cuh"
 
 namespace mpd {

@@ -19,14 +19,16 @@
 // one barrier per exchange is enough: a buffer is rewritten only after the barrier that follows
 // the reads of it.  S is as large as the lanes allow (a chunk of 16 cells: two steps of the
 // two-pass scheme with the limiter).  A system's equations are coupled per cell, so each warp
-// advects one equation's chunk and every step exchanges.
+// advects one equation's chunk and every step exchanges.  Each block gets as few warps as hold its
+// cells (500 cells: 16 blocks of 2).
 //
 // The arithmetic is that of the staged kernels (same expressions); each face's flux is formed
 // once and shuffled to the cell on its right.
 //
-// Measured: 500 cells, FP64, two passes with the limiter 11.2 -> 2.2 us per step (one warp per SM
-// sub-partition; 36 FP64 instructions per step at about 70 clocks each, then the barrier); the
-// FP64 system of two equations and 1000 cells 58 -> 4.2 us per step.
+// Measured: 500 cells, FP64, two passes with the limiter 11.2 -> 2.1 us per step, of which the chain
+// of 36 dependent FP64 instructions at about 70 clocks each takes 1.2 and the exchange every second
+// step and the idle sub-partitions (two warps on four) the rest; the FP64 system of two equations
+// and 1000 cells 58 -> 4.0 us per step (six warps on four sub-partitions, an exchange every step).
 #include <cuda_runtime.h>
 
 #include "internal.h"
@@ -349,7 +351,8 @@ template <typename T>
 int line1d_steps(const Grid& g, const Opts& o, const T* psi_in, T* psi_out, const T* gc, const T* G, const T* R, T dt,
                  int n_steps, const TrapezMat* m, const T* b, bool chained, cudaStream_t st) {
   if (g.nd != 1 || o.dfl || o.open) return MPDATA_EUNSUPPORTED;
-  // FP64 |psi| stays on the staged kernels: on a positive field it is their basic scheme bit for bit
+  // FP64 |psi| stays on the staged kernels (k_steps1d): the option's step on a positive field is to have
+  // the bits of the basic step there (MPDATA_STAGED), and the products here are contracted differently
   if (o.abs && sizeof(T) == 8) return MPDATA_EUNSUPPORTED;
   if (g.N > (1 << 20) || o.n_iters > 64) return MPDATA_EUNSUPPORTED;
   LineParams<T> p{};

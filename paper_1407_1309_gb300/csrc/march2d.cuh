@@ -2,7 +2,8 @@
 // pseudo-advector (Eq. 6 with its cross term), the FCT limiting factors and the
 // corrective donor-cell pass of one time step in one kernel, with no
 // intermediate written to global memory.  Covers 2D fields with n_iters = 2 and
-// every option except the third-order terms and open edges (those run on the staged path).
+// every option except the third-order terms and open edges (tile2d.cu or the staged kernels), in FP64
+// also except |psi| and the divergent-flow term.
 //
 // Work decomposition ("warp march"): a warp owns a strip of 32*NC columns (NC
 // adjacent columns per lane) and walks down TY rows.  Vertical neighbours stay
@@ -85,7 +86,7 @@ __device__ __forceinline__ void march_tile(const F2Params<T>& p, const int strip
   constexpr int kCols = cols<NC>();
   constexpr int kStride = stride<NC>();
   constexpr bool DFL = (EXT & kExtDfl) != 0;
-  // psi as it enters the psi-fractions (|psi| with the variable-sign option: an operand modifier)
+  // psi as it enters the psi-fractions (|psi| with the variable-sign option)
   auto fr = [](const T x) { return (EXT & kExtAbs) ? absv(x) : x; };
   const int lc0 = NC * lane;
   const int cs = strip * kStride - kLead;

@@ -20,29 +20,32 @@ template <typename T> __device__ __forceinline__ T fdiv(T a, T b);
 // FP32 n / d (2 ulp), also for a d below the smallest normal number: the limiter divides by flux
 // sums, which become that small in the tail of a field.
 template <> __device__ __forceinline__ float fdiv<float>(float a, float b) { return __fdividef(a, b); }
-// Approximate FP32 reciprocals.  rcp() takes and gives subnormal numbers; rcp_normal() flushes them to
-// zero and is for a divisor known to be normal whose quotient is 0 above 2^126, as __fdividef's is
-// (the psi-fractions: divisible()).
-__device__ __forceinline__ float rcp(float d) {
-  float r;
-  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(d));
-  return r;
-}
+// Approximate FP32 reciprocal of a divisor known to be normal (the psi-fractions: divisible()), in
+// which subnormal numbers are flushed: 0 above 2^126, as __fdividef's quotient is.
 __device__ __forceinline__ float rcp_normal(float d) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
   return r;
 }
+// Approximate FP32 reciprocal that takes and gives subnormal numbers: of d scaled by a power of two
+// into the range of the form above (PTX's rcp.approx.f32 in its place: 256^3 with three passes and
+// third-order terms 1086 -> 1100 us per step).
+__device__ __forceinline__ float rcp(float d) {
+  const float s = fabsf(d) > 1.0f ? 0.25f : 16777216.0f;
+  return rcp_normal(d * s) * s;
+}
+
 // FP64 n / d for the arithmetic-bound FP64 kernels, five FP64 operations: one Newton-Raphson
 // iteration r <- r + r (1 - d r) (quadratic convergence) from the PTX approximate FP64 reciprocal
 // (rcp.approx.ftz.f64, full exponent range), and Markstein's remainder correction
 // q <- q + r (n - d q) of the quotient: within one unit in the last place of the exact quotient for
-// normal operands.  The seed carries about 20 bits, the iterated reciprocal 40; the remainder is
-// exact in the fma, so the corrected quotient's error before its last rounding is the product of
-// two 2^-40 errors.  Measured against IEEE division: all of 4 10^8 quotients equal, with this
-// form and with a second iteration alike; without it the 1024^2 FP64 step takes 215 instead of
-// 242 us.  A zero, infinite or NaN divisor gives NaN (the kernels never rely on it: the psi-ratio guards zero sums, and the FCT
-// factors' min(1, x) maps the inf or NaN of a zero flux sum to 1 alike).
+// normal operands.  The seed carries about 20 bits, the iterated reciprocal 40, and so does the first
+// quotient; the fma rounds its remainder to 53 bits of a correction of relative size 2^-40, so that
+// the corrected quotient's error before its last rounding is about 2^-80.  Measured against IEEE
+// division: none of 4 10^8 quotients differs, with this form and with a second iteration alike;
+// without that the 1024^2 FP64 step takes 215 instead of 242 us.  A zero, infinite or NaN divisor
+// gives NaN (the kernels never rely on it: the psi-ratio guards zero sums, and the FCT factors'
+// min(1, x) maps the inf or NaN of a zero flux sum to 1 alike).
 __device__ __forceinline__ double nr_div(double n, double d) {
   double r0;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(d));
@@ -57,18 +60,19 @@ template <typename T> __device__ __forceinline__ T negp(T x) { return x < T(0) ?
 template <typename T> __device__ __forceinline__ T absv(T x) { return x < T(0) ? -x : x; }
 template <typename T> __device__ __forceinline__ T maxv(T a, T b) { return a > b ? a : b; }
 template <typename T> __device__ __forceinline__ T minv(T a, T b) { return a < b ? a : b; }
-// FP32: one min/max instruction (the ternary forms compile to a compare and a select, both on
-// the half-rate ALU pipe, to keep the ternary's choice for NaN), |x| as an operand modifier.
-// The 2D and 3D marches are bound by issue and the ALU pipe; these forms, the three-value extrema
-// and the flushing reciprocal together, same bits, measured per step: 4096^2 139 -> 104 us, the
-// compensated 1024^2 18.4 -> 15.0 us, the 512-field ensemble 539 -> 400 us, 256^3 with three
-// passes and third-order terms 1248 -> 1050 us.
+// FP32: PTX min and max, which return the number where one operand is NaN (the ternary forms have
+// to return a particular operand then), and |x|.  The 2D and 3D marches are bound by issue and the
+// half-rate ALU pipe that runs comparisons and selections; these forms, the three-value extrema
+// below, selected upwind values and the flushing reciprocal of the guarded psi-fractions together,
+// measured per step: 4096^2 139 -> 90 us (with the tile heights of lanes2d.h), the compensated
+// 1024^2 18.4 -> 13.2 us, the 512-field ensemble 539 -> 402 us, 256^3 with three passes and
+// third-order terms 1248 -> 1086 us.
 template <> __device__ __forceinline__ float posp<float>(float x) { return fmaxf(x, 0.0f); }
 template <> __device__ __forceinline__ float negp<float>(float x) { return fminf(x, 0.0f); }
 template <> __device__ __forceinline__ float absv<float>(float x) { return fabsf(x); }
 template <> __device__ __forceinline__ float maxv<float>(float a, float b) { return fmaxf(a, b); }
 template <> __device__ __forceinline__ float minv<float>(float a, float b) { return fminf(a, b); }
-// extrema of three values: one instruction in FP32
+// extrema of three values: PTX's three-operand min and max in FP32
 template <typename T> __device__ __forceinline__ T max3(T a, T b, T c) { return maxv(maxv(a, b), c); }
 template <typename T> __device__ __forceinline__ T min3(T a, T b, T c) { return minv(minv(a, b), c); }
 template <> __device__ __forceinline__ float max3<float>(float a, float b, float c) {

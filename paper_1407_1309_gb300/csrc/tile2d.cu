@@ -345,8 +345,9 @@ int launch_tile(const TileParams<T>& p, int fields, bool always, cudaStream_t st
 template <typename T>
 int tile2d_step(const Grid& g, const Opts& o, const StepArgs<T>& a, int fields, long long field, cudaStream_t st) {
   if (g.nd != 2 || o.n_iters < 2 || o.n_iters > 8 || a.psi_in == a.psi_out) return MPDATA_EUNSUPPORTED;
-  // periodic FP64 |psi| without the divergent-flow term stays on the staged kernels: on a positive
-  // field it is their basic scheme bit for bit, and contraction differs between the two
+  // periodic FP64 |psi| without the divergent-flow term stays on the staged kernels: its step on a
+  // positive field is to have the bits of the basic step there (MPDATA_STAGED), and the products here
+  // are contracted differently
   if (sizeof(T) == 8 && o.abs && !o.dfl && !o.open) return MPDATA_EUNSUPPORTED;
   TileParams<T> p;
   p.psi = a.psi_in;
