@@ -17,7 +17,7 @@ constexpr int strip_stride(int nc) { return 32 * nc - 2 * kLead; }
 // SM at k blocks, for the k of least time, even (the march's loop takes two rows a turn, and its
 // single last row of an odd height rounds the products differently, so that a result would depend
 // on the height); a field with more strips than that has warps is not cut into rows.  Against the earlier list of heights (the tallest with 7.5 warps per SM): 4096^2
-// 102 -> 90 us (80 rows instead of 64), 2000 x 500 13.9 -> 10.8 us (with lanes of 2).
+// 102 -> 90 us (80 rows instead of 64), 2000 x 500 13.9 -> 10.3 us (with lanes of 2).
 struct MarchRows {
   int ty;
   float us;
@@ -47,7 +47,7 @@ inline MarchRows march_rows(int nc, int n0, int n1, bool comp) {
 
 // Whether lanes of 2 columns suit an FP32 field better than lanes of 4: where the narrower strips
 // leave fewer padded columns or, on a field too small to fill the GPU, their twice as many warps
-// hide more latency (compensated 512^2 12.1 -> 8.1 us, plain 2000 x 500 13.9 -> 10.8).
+// hide more latency (compensated 512^2 12.1 -> 7.4 us, plain 2000 x 500 13.9 -> 10.3).
 inline bool narrow_lanes(int n0, int n1, bool comp) {
   return march_rows(2, n0, n1, comp).us < 0.98f * march_rows(4, n0, n1, comp).us;
 }

@@ -16,7 +16,7 @@ inline long long march3_blocks(const int (&n)[3], int nc, int zc) {
 // z-planes per block, 4 to 16: the chunk of least time by the load of the fullest SM.  A block takes
 // about zc + 3 plane steps (its halo planes are staged, pass 1 and the factors recomputed on two of
 // them); two blocks share an SM and take 1.5 times as long as one there.  Large fields get 16
-// (measured at 256^3: 8 .. 24 within 2 %); 128^3, one block per SM with 16, gets 7 and two: 206 -> 151
+// (measured at 256^3: 8 .. 24 within 2 %); 128^3, one block per SM with 16, gets 7 and two: 206 -> 144
 // us per step of three passes with third-order terms.  steps: the plane steps of the fullest SM, in units of
 // those of one block alone.
 struct ZChunk {

@@ -5,8 +5,8 @@
 // columns; march3_form).
 //
 // Against the scalar z-marches of staged.cu, whose threads own one cell each: 101 x 97 x 103 with
-// three passes, third-order terms, limiter and G 233 -> 149 us per step, 64^3 133 -> 59,
-// 256 x 256 x 255 1743 -> 1347 (256^3 with 16-byte chunks 1061).
+// three passes, third-order terms, limiter and G 233 -> 142 us per step, 64^3 133 -> 49,
+// 256 x 256 x 255 1743 -> 1369 (256^3 with 16-byte chunks 1088).
 #include "march3.cuh"
 
 namespace mpd {
